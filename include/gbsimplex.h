@@ -133,10 +133,16 @@ typedef struct {
     int pipeline;            /* single-LP primal simplex kernel:
                                 0 = selection, then update (one launch-wide
                                     grid barrier per pivot);
-                                1 = auto (default): 2 below 2^19 tableau
-                                    elements ((m+1) x row pitch), else 4; 2
-                                    when the second buffer cannot be
-                                    allocated;
+                                1 = auto (default): the panel kernel, for the
+                                    primal and the dual rule: pivots are
+                                    selected on rows and columns formed on
+                                    demand and applied to the tableau, in
+                                    place, up to 16 at a time; where it cannot
+                                    take the LP (its workspace or its shared
+                                    memory does not fit) or n > 4 m from 2^20
+                                    tableau elements on, 2 below 2^19 elements
+                                    ((m+1) x row pitch), else 4 (2 when the
+                                    second buffer cannot be allocated);
                                 2 = pipelined in place: the next pivot's
                                     selection overlaps this pivot's update, no
                                     grid barrier;
@@ -149,8 +155,8 @@ typedef struct {
                                     CTA forms the new pivot columns on its own
                                     rows and the ratio test is distributed;
                                 5 = as 4, the ratio test always distributed.
-                                The dual rule (LP_MIN_GE, and FP32 recovery)
-                                always runs double-buffered: one pivot per pass
+                                Otherwise the dual rule (LP_MIN_GE, and FP32
+                                recovery) runs double-buffered: one pivot per pass
                                 for 2 and 3, two for 1, 4 and 5.
                                 Same pivots and bits in every mode.              */
     long long solo_elems;    /* servers: an LP of at least this many tableau
@@ -182,8 +188,13 @@ typedef struct {
                                 FP32 body does not build up; 0 = only the rhs,
                                 the duals and the objective row.  Batches do
                                 the latter.                                     */
-    int zero_skip;           /* two-pivot primal kernel (pipeline 1, 4, 5: the
-                                primal rule, FP64 or the FP32 tableau), on
+    int zero_skip;           /* panel kernel (pipeline 1): 1 (default, where
+                                m >= n / 4) and 2 = a panel leaves out the
+                                columns that are basic throughout it, whose
+                                entries in its pivot rows are zeros; 0 = it
+                                updates every column.  Two-pivot primal
+                                kernel (pipeline 4, 5, and where 1 takes it:
+                                the primal rule, FP64 or the FP32 tableau), on
                                 tableaus of at least 2^25 elements ((m+1) x row
                                 pitch) with m >= n / 4: 1 (default) = each CTA owns a
                                 run of the structural columns and one of the
@@ -413,7 +424,8 @@ lp_err lp_solve_noalloc(int m, int n, const double *A, const double *b, const do
                         lp_sense sense, const lp_options *opt, double *x, double *y,
                         double *obj, lp_status *status, long long *iters);
 
-/* Constraint-row entries the two-pivot primal kernel updated (*updated,
+/* Constraint-row entries the panel kernel and the two-pivot primal kernel
+ * updated (*updated,
  * each read, updated and written) and left in place (*in_place, see
  * lp_options.zero_skip), in 16-byte vectors times pivots, summed over the
  * solves since lp_load (the objective row, always updated, not counted).

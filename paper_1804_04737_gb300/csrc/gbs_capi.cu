@@ -70,13 +70,16 @@ struct lp_handle {
     size_t cap_T2 = 0;
     void *dcolx = nullptr;                      // two-pivot kernel: four pivot-column slots
     size_t cap_colx = 0;
+    void *dpanel = nullptr;                     // panel kernel: pending columns and rows
+    size_t cap_panel = 0;
     int *dbasis = nullptr;
     size_t cap_basis = 0;
     void *dscratch = nullptr;
     size_t cap_scratch = 0;                     // bytes
     Cand *dpart = nullptr;                      // 38 * max_ctas (records, values)
     int max_ctas = 0;
-    unsigned *dbar = nullptr;                   // kBarWords: barrier, counters, err
+    unsigned *dbar = nullptr;                   // kBarWords: barrier, counters, err; then the
+                                                // panel kernel's records and the update counts
     int *dtrace = nullptr;
     long long cap_trace = 0;
     LpDesc *ddesc = nullptr;
@@ -269,8 +272,9 @@ lp_err lp_create(lp_handle **out, const lp_options *opt) {
     }
     if (e == cudaSuccess) e = cudaMalloc(&h->ddesc, sizeof(LpDesc));
     if (e == cudaSuccess) e = cudaMalloc(&h->dstats, sizeof(InputStats));
-    // the synchronisation block, then the two-pivot kernels' update counts
-    if (e == cudaSuccess) e = cudaMalloc(&h->dbar, (kBarWords + 4) * sizeof(unsigned));
+    // the synchronisation block, the panel kernel's records, the update counts
+    if (e == cudaSuccess)
+        e = cudaMalloc(&h->dbar, (kBarWords + kPanelRecWords + 4) * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc(&h->dobj, sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&h->pdesc, sizeof(LpDesc));
     if (e == cudaSuccess) e = cudaMallocHost(&h->pobj, sizeof(double));
@@ -299,7 +303,7 @@ void lp_destroy(lp_handle *h) {
                      h->rb.pivrow, h->rb.W, h->rb.xS, h->rb.yR, h->rb.zrow, h->rb.rhs, h->rb.chk,
                      h->rb.bar};
     for (void *p : rbufs) dev_free(h, p);
-    void *grown[] = {h->dA, h->db, h->dc, h->dT, h->dT2, h->dcolx, h->dbasis, h->dscratch,
+    void *grown[] = {h->dA, h->db, h->dc, h->dT, h->dT2, h->dcolx, h->dpanel, h->dbasis, h->dscratch,
                      h->dpart, h->dtrace, h->dx, h->dy};
     for (void *p : grown) dev_free(h, p);
     void *bufs[] = {h->dbar, h->ddesc, h->dstats, h->dobj};
@@ -382,7 +386,29 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     if (pmode == 5) pmode = 4;
     const size_t tbytes = (size_t)M * P * esz;
     if (pmode == 1) pmode = (long long)M * P >= kBlockElems ? 4 : 2;
-    const bool dwant = dualr && h->opt.pipeline != 0;
+    // The automatic mode takes the panel kernel for every rule the LP needs,
+    // where its shared memory and its workspace fit (a workspace above 64 MB
+    // only when the tableau is at least twice as large); then no second
+    // buffer is needed.  Not on wide LPs above 2^20 elements: every vector is
+    // updated there, and a CTA's few rows split unevenly (512 x 4096: 11.0 us
+    // per pivot against 10.8).
+    const int pdrop = h->opt.zero_skip == 2 || (h->opt.zero_skip == 1 && 4ll * m >= n);
+    const size_t pws = panel_workspace(h->prec, m, P);
+    bool panel = h->opt.pipeline == 1 &&
+                 (4ll * m >= n || (long long)M * P < (1ll << 20)) && (pws <= (64ull << 20) || 2 * pws <= tbytes) &&
+                 choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, (int)sense, pdrop).pipe == 4;
+    if (panel && h->region) {
+        // (what the buffers below take besides the inputs, with slack)
+        const size_t need = tbytes + pws + (size_t)(m + n) * 16 +
+                            64 * (size_t)h->sms * sizeof(Cand) + (64u << 10);
+        panel = h->region_size - h->region_used >= need;
+    }
+    if (panel && grow_bytes(h, &h->dpanel, &h->cap_panel, pws) != cudaSuccess) {
+        cudaGetLastError();
+        panel = false;
+    }
+    if (panel) pmode = 0;
+    const bool dwant = dualr && h->opt.pipeline != 0 && !panel;
     bool have_t2 = false;
     if (pmode >= 3 || dwant) {
         have_t2 = grow_bytes(h, &h->dT2, &h->cap_T2, (size_t)M * P * esz) == cudaSuccess;
@@ -411,6 +437,8 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     const int sector = h->prec == PREC_FP64 ? 4 : 8;
     const int split = skip ? n / sector * sector : 0;
     auto shape_for = [&](int rule) {
+        if (panel)
+            return choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, rule, pdrop);
         if (rule == 0 && pmode) {
             PivotShape ps = choose_pipe_shape(h->prec, M, P, h->sms, h->opt.threads, h->opt.ctas,
                                               pmode == 4 ? 2 : 0, pmode == 4 ? split : 0);
@@ -522,8 +550,9 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     d.part_vals = reinterpret_cast<unsigned long long *>(h->dpart + 4 * (size_t)h->max_ctas);
     d.T2 = have_t2 ? h->dT2 : nullptr;
     d.colx = h->dcolx;
-    d.abort = h->dabort;
-    d.work = reinterpret_cast<unsigned long long *>(h->dbar + kBarWords);
+    d.panel = h->dpanel;
+    d.abort = h->opt.time_limit_s > 0.0 ? h->dabort : nullptr;
+    d.work = reinterpret_cast<unsigned long long *>(h->dbar + kBarWords + kPanelRecWords);
     CUDA_TRY(h, cudaMemsetAsync(d.work, 0, 2 * sizeof(unsigned long long), s));
     // a constraint row may hold a -0: from the data, after Phase 1 (dual
     // pivots are negative), or in FP32 mode once a reinversion has rewritten
@@ -569,6 +598,12 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
 }  // extern "C"
 
 namespace {
+
+// The words a pivot launch wants zeroed: the synchronisation block, and the
+// records of the panel kernel.
+size_t bar_bytes(const PivotShape &sh) {
+    return (kBarWords + (sh.pipe == 4 ? kPanelRecWords : 0)) * sizeof(unsigned);
+}
 
 // Start the wall-clock limit of a solve: lower the abort word (no kernel of
 // this handle is running: the previous solve was waited for) and set the
@@ -729,7 +764,7 @@ lp_err solve_fp32(lp_handle *h) {
         const long long stride = sh.scratch_stride;
         CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, scratch_stride), &stride,
                                     sizeof stride, cudaMemcpyHostToDevice, s));
-        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, kBarWords * sizeof(unsigned), s));
+        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape_alt), s));
         CUDA_TRY(h, cudaEventRecord(h->ev0, s));
         CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, sh, h->opt.spin_timeout_cycles, budget, s));
         CUDA_TRY(h, cudaEventRecord(h->ev1, s));
@@ -835,7 +870,7 @@ lp_err lp_solve_async(lp_handle *h) {
         // objective row is max(-c, 0), until no rhs is below -eps_r.  The
         // host waits for its end to choose what follows.
         const long long before = h->pdesc->iters;
-        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, kBarWords * sizeof(unsigned), s));
+        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
         CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, h->shape_alt, h->opt.spin_timeout_cycles,
                                  budget, s));
         CUDA_TRY(h, cudaMemcpyAsync(h->pdesc, h->ddesc, sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
@@ -867,7 +902,7 @@ lp_err lp_solve_async(lp_handle *h) {
             return LP_OK;
         }
     }
-    CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, kBarWords * sizeof(unsigned), s));
+    CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
     CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, h->shape, h->opt.spin_timeout_cycles, budget, s));
     CUDA_TRY(h, cudaEventRecord(h->ev1, s));
     CUDA_TRY(h, launch_extract(h->prec, h->ddesc, h->dT, h->dbasis, h->m, h->n, h->P, h->sense,
@@ -917,7 +952,7 @@ lp_err lp_update_counts(lp_handle *h, long long *updated, long long *in_place) {
     CUDA_TRY(h, cudaSetDevice(h->device));
     CUDA_TRY(h, wait_stream(h));
     unsigned long long v[2] = {0ull, 0ull};
-    CUDA_TRY(h, cudaMemcpy(v, h->dbar + kBarWords, sizeof v, cudaMemcpyDeviceToHost));
+    CUDA_TRY(h, cudaMemcpy(v, h->dbar + kBarWords + kPanelRecWords, sizeof v, cudaMemcpyDeviceToHost));
     // the kernels count vectors x pivots; a vector is 16 bytes of one row,
     // over the m constraint rows
     const long long per = (long long)(h->prec == PREC_FP64 ? 2 : 4) * h->m;
@@ -1040,7 +1075,7 @@ lp_err handle_bind_region(lp_handle *h, void *base, size_t bytes) {
     cudaSetDevice(h->device);
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     void **bufs[] = {(void **)&h->dA, (void **)&h->db, (void **)&h->dc, &h->dT, &h->dT2,
-                     &h->dcolx, (void **)&h->dbasis, &h->dscratch, (void **)&h->dpart,
+                     &h->dcolx, &h->dpanel, (void **)&h->dbasis, &h->dscratch, (void **)&h->dpart,
                      (void **)&h->dtrace, (void **)&h->dx, (void **)&h->dy,
                      (void **)&h->rb.Lflag, (void **)&h->rb.S, (void **)&h->rb.R,
                      (void **)&h->rb.posS, (void **)&h->rb.posR, (void **)&h->rb.counts,
@@ -1051,7 +1086,7 @@ lp_err handle_bind_region(lp_handle *h, void *base, size_t bytes) {
         dev_free(h, *p);
         *p = nullptr;
     }
-    h->cap_A = h->cap_b = h->cap_c = h->cap_T = h->cap_T2 = h->cap_colx = 0;
+    h->cap_A = h->cap_b = h->cap_c = h->cap_T = h->cap_T2 = h->cap_colx = h->cap_panel = 0;
     h->cap_basis = h->cap_scratch = h->cap_x = h->cap_y = 0;
     h->max_ctas = 0;
     h->cap_trace = 0;

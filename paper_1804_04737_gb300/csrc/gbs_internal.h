@@ -76,6 +76,8 @@ struct LpDesc {
     // nonzero when a constraint row may hold a -0 (from the data, Phase I,
     // FP32 mode, or a -0 an update produced): no vector is left in place
     int negz;
+    // panel kernel: its pending columns and rows (panel_workspace bytes)
+    void *panel;
 };
 
 // Launch shape of the persistent pivot kernel for one LP.
@@ -85,11 +87,13 @@ struct PivotShape {
     int strip = 0;                 // columns per strip (multiple of 32 bytes of elements)
     int use_smem = 0;              // selection scratch in shared memory (else global)
     int dual = 0;                  // dual simplex kernel (else primal)
-    int pipe = 0;                  // pipelined kernel: 1 in place, 2 double-buffered, 3 two pivots per pass
+    int pipe = 0;                  // pipelined kernel: 1 in place, 2 double-buffered, 3 two pivots per pass,
+                                   // 4 the panel kernel
     int sel_warps = 4;             // two pivots per pass: selection warps per CTA (4 or 8)
     int dist = 0;                  // two pivots per pass, primal: ratio test distributed over the CTAs
     int split = 0;                 // two pivots per pass, primal: first column of every CTA's second
                                    // run (0: one contiguous strip, every vector updated)
+    int drop = 0;                  // panel kernel: leave out columns that stay basic
     size_t smem_bytes = 0;         // dynamic shared memory per CTA
     long long scratch_stride = 0;  // global scratch bytes per CTA when !use_smem
 };
@@ -102,6 +106,14 @@ struct PivotShape {
 // kernels), [192] ratio-records counter and [224] exact-rounds counter
 // (two-pivot primal kernel); 128-byte apart.
 constexpr int kBarWords = 256;
+
+// The panel kernel (gbs_panel.cu): pivots pending at most, CTA size, and CTAs
+// at most.  Its two record exchanges (a 128-byte line per CTA and exchange) follow
+// the synchronisation block and are zeroed with it before each launch.
+constexpr int kPanelK = 16;
+constexpr int kPanelThreads = 256;
+constexpr int kPanelMaxCtas = 192;
+constexpr int kPanelRecWords = 2 * kPanelMaxCtas * 32;
 
 struct InputStats {
     unsigned long long amax_bits, bmax_bits, cmax_bits;  // bit patterns of max |.|
@@ -150,6 +162,12 @@ PivotShape choose_pipe_shape(int prec, int M, long long P, int sms, int threads,
                              int dual, int split = 0);
 cudaError_t launch_pivot_pipe(int prec, LpDesc *d_desc, const PivotShape &sh,
                               long long spin_limit, long long budget, cudaStream_t s);
+// The panel kernel's shape (pipe == 0: its shared memory does not fit), its
+// workspace bytes and its launch (gbs_panel.cu).
+PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop);
+size_t panel_workspace(int prec, int m, long long P);
+cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
+                         long long budget, cudaStream_t s);
 cudaError_t launch_extract(int prec, const LpDesc *d_desc, const void *T, const int *basis,
                            int m, int n, long long P, int sense, double *x, double *y,
                            double *obj, cudaStream_t s);

@@ -1,0 +1,88 @@
+"""GPU: the panel kernel (the default of single solves) at the edges of its split.
+
+Each CTA owns a slice of the rows and a strip of the columns, selects on
+entries formed on demand and applies up to 16 pending pivots at a time; the
+pivots and every bit of the tableau must be the oracle's where slices are
+empty, uneven or one element wide, where a call ends inside, at the end or
+just after a panel, in both forms, with basic columns left out of the panels
+and without, and where the ratios' single-precision keys leave their range.
+"""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1804_04737_gb300 import capi, lpgen
+from paper_1804_04737_gb300.build import build_library
+from test_gpu_parity import Run, _bits, _oracle, assert_same
+
+pytestmark = pytest.mark.gpu
+
+MAX_LE, MIN_GE = capi.LP_MAX_LE, capi.LP_MIN_GE
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_library()
+    capi.load_library()
+    oracle.set_threads(os.cpu_count() or 1)
+    yield
+    oracle.set_threads(1)
+
+
+@pytest.mark.parametrize("zero_skip", [0, 1, 2])
+@pytest.mark.parametrize("sense", [MAX_LE, MIN_GE])
+@pytest.mark.parametrize("m,n,ctas", [(1, 1, 0), (2, 1, 0), (1, 40, 0), (40, 1, 0), (17, 33, 5),
+                                      (31, 32, 152), (130, 90, 152), (305, 40, 1), (40, 305, 1),
+                                      (305, 700, 2), (611, 310, 0), (90, 2600, 9)])
+def test_slices_bitwise(m, n, ctas, sense, zero_skip):
+    for A, b, c in (lpgen.dense_lp(m, n, seed=m + n), lpgen.paper_lp(m, n, seed=m + n)):
+        if sense == MIN_GE:
+            A, b, c = lpgen.dual_of(A, b, c)
+            c = np.abs(c)
+        assert_same(Run(A, b, c, sense, ctas=ctas, zero_skip=zero_skip, time_limit_s=60.0),
+                    _oracle(A, b, c, sense))
+
+
+@pytest.mark.parametrize("chunk", [1, 15, 16, 17, 33])
+@pytest.mark.parametrize("kind", ["primal", "dual", "phase1"])
+def test_calls_that_end_around_a_panel(chunk, kind):
+    """Resumed in calls of `chunk` pivots: each call applies what is pending,
+    so the next one starts from the tableau alone."""
+    A, b, c = lpgen.paper_lp(150, 170, seed=4) if kind != "phase1" else lpgen.dense_lp(120, 90, seed=1)
+    sense = MAX_LE
+    if kind == "dual":
+        A, b, c = lpgen.dual_of(A, b, c)
+        sense = MIN_GE
+    if kind == "phase1":
+        A, b = lpgen.with_ge_rows(A, b, 0.1, seed=2)
+    o = _oracle(A, b, c, sense)
+    m, n = A.shape
+    h = capi.lp_create(capi.lp_options_default(max_iters=chunk))
+    try:
+        capi.lp_load(h, A, b, c, sense)
+        for _ in range(o.iters + 2):
+            capi.lp_solve(h)
+            x, y = np.empty(n), np.empty(m)
+            obj, st, it = capi.lp_result(h, x, y)
+            if st != capi.LP_ITER_LIMIT:
+                break
+        assert st == o.status and it == o.iters and _bits([obj])[0] == _bits([o.obj])[0]
+        assert np.array_equal(_bits(x), _bits(o.x)) and np.array_equal(_bits(y), _bits(o.y))
+        assert np.array_equal(_bits(capi.lp_get_tableau(h, m, n)), _bits(o.T))
+    finally:
+        capi.lp_destroy(h)
+
+
+@pytest.mark.parametrize("sense", [MAX_LE, MIN_GE])
+@pytest.mark.parametrize("e", [40, 61, 200])
+def test_ratio_keys_out_of_range(e, sense):
+    """Rows and columns scaled by 2^+-e: all, some or none of the ratios'
+    operands lie within the keys' range of exponents (2^+-60)."""
+    from test_gpu_scaled import scaled_lp
+    (A, b, c), eps, _ = scaled_lp(90, 110, e, seed=e)
+    if sense == MIN_GE:
+        A, b, c = lpgen.dual_of(A, b, c)
+        eps = {"eps_d": eps["eps_r"], "eps_p": eps["eps_p"], "eps_r": eps["eps_d"]}
+    assert_same(Run(A, b, c, sense, zero_skip=2, **eps), _oracle(A, b, c, sense, **eps))
