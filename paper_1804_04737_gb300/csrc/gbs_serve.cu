@@ -351,6 +351,27 @@ double *pin_take(lp_server *sv, size_t bytes, int *cls) {
     return static_cast<double *>(p);
 }
 
+// The pool's first buffers, from one allocation when the server starts: 32 of
+// each class up to 64 KiB (4 MiB).  A host allocation waits behind the kernels
+// in flight, so without them the first small requests behind a large LP were
+// not queued before it had ended.
+constexpr int kPinFirst = 32, kPinFirstLo = 12, kPinFirstHi = 16;
+cudaError_t pin_prefill(lp_server *sv) {
+    size_t bytes = 0;
+    for (int k = kPinFirstLo; k <= kPinFirstHi; ++k) bytes += kPinFirst * ((size_t)1 << k);
+    void *p = nullptr;
+    cudaError_t e = cudaHostAlloc(&p, bytes, cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    sv->pin_all.push_back(p);
+    sv->pin_total += bytes;
+    sv->pin_free.resize(kPinFirstHi + 1);
+    unsigned char *at = static_cast<unsigned char *>(p);
+    for (int k = kPinFirstHi; k >= kPinFirstLo; --k)  // largest first: each stays aligned to its size
+        for (int i = 0; i < kPinFirst; ++i, at += (size_t)1 << k)
+            sv->pin_free[k].push_back(reinterpret_cast<double *>(at));
+    return cudaSuccess;
+}
+
 // The request's pinned inputs back to the pool (their copy to the device is
 // complete, or they are not needed any more).
 void pin_give(lp_server *sv, Request &r) {
@@ -1289,6 +1310,7 @@ lp_err lp_server_create(lp_server **out, const lp_options *opt, size_t hbm_budge
     if (e == cudaSuccess) e = cudaMalloc(&sv->d_ctl, sizeof(ServeCtl));
     if (e == cudaSuccess) e = cudaHostAlloc(&sv->h_ring, sizeof(ServeRing), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&sv->d_ring, sv->h_ring, 0);
+    if (e == cudaSuccess) e = pin_prefill(sv);
     if (e == cudaSuccess && sv->fp32) {
         // the batched FP32 launches: a strip of up to threads * 4 floats, the
         // pivot column (FP32) and an FP64 row of the LP's width per CTA
