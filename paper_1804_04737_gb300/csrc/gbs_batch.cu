@@ -9,8 +9,13 @@
 // and a 32 x 32 LP finish in comparable times.  Device memory is kept in a
 // per-device grow-only pool between calls.
 //
-// Per-LP arithmetic is exactly the single-LP kernel's (same device function),
-// so every LP's pivots and results are bit for bit those of solving it alone.
+// Per-LP arithmetic is exactly the single-LP kernel's (same device function,
+// panel_solve), so every LP's pivots and results are bit for bit those of
+// solving it alone.  Two CTAs of 256 threads per SM: one LP's selection chain
+// runs under another's panels.  1024 LPs of 32 to 1024 rows and columns: the
+// pivot kernel takes 5.8 ms (24 with the kernel that updates the tableau every
+// pivot; 5.6 ms is the FP64 time of the columns that change), at 262144 tableau
+// elements per CTA (6.7 ms at 131072, 8.9 at 524288); FP32 rounds 2.1 ms (8).
 
 #include <cuda_runtime.h>
 #include <stdarg.h>
@@ -29,6 +34,9 @@ namespace gbs {
 namespace {
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Dynamic shared memory of a batched panel CTA, two per SM.
+constexpr size_t kPanelBatchSmem = 104 * 1024;
 
 // ---------------------------------------------------------------- kernels --
 
@@ -242,8 +250,8 @@ struct BatchFp32 {
     int2 *h_items, *d_items;
     unsigned *d_queue;
     unsigned char *d_bar;
-    int ctas, threads, use_smem, sms;
-    size_t smem;
+    int ctas, threads, use_smem, sms, panel, drop;
+    size_t smem, bar_bytes;
     const lp_options *opt;
     cudaStream_t s;
 };
@@ -291,16 +299,23 @@ lp_err solve_batch_fp32(const BatchFp32 &f, lp_status *fin, double *kernel_ms) {
             budget = std::min(budget, remaining[k]);
             for (int r = 0; r < f.G[k]; ++r) f.h_items[nitems++] = make_int2(k, r);
             f.h_desc[k].sense = rule[k];
+            // (the dual rule's negative pivots leave -0 in basic columns)
+            if (rule[k]) f.h_desc[k].negz = 1;
             before[k] = f.h_desc[k].iters;
         }
         if (nitems == 0) break;
         B_TRY(cudaMemcpyAsync(f.d_items, f.h_items, nitems * sizeof(int2), cudaMemcpyHostToDevice, s));
         B_TRY(cudaMemcpyAsync(f.d_desc, f.h_desc, count * sizeof(LpDesc), cudaMemcpyHostToDevice, s));
-        B_TRY(cudaMemsetAsync(f.d_bar, 0, (size_t)count * 512, s));
+        B_TRY(cudaMemsetAsync(f.d_bar, 0, f.bar_bytes, s));
         B_TRY(cudaMemsetAsync(f.d_queue, 0, sizeof(unsigned), s));
         B_TRY(cudaEventRecord(e0, s));
-        B_TRY(launch_batch(PREC_FP32, f.d_desc, f.d_items, nitems, f.d_queue, f.ctas, f.threads,
-                           f.smem, f.use_smem, f.opt->spin_timeout_cycles, budget, s));
+        if (f.panel)
+            B_TRY(launch_panel_batch(PREC_FP32, f.d_desc, f.d_items, nitems, f.d_queue, f.ctas,
+                                     f.smem, f.opt->spin_timeout_cycles, budget, f.drop, s));
+        else
+            B_TRY(launch_batch(PREC_FP32, f.d_desc, f.d_items, nitems, f.d_queue, f.ctas,
+                               f.threads, f.smem, f.use_smem, f.opt->spin_timeout_cycles, budget,
+                               s));
         B_TRY(cudaEventRecord(e1, s));
         B_TRY(cudaMemcpyAsync(f.h_desc, f.d_desc, count * sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
         B_TRY(cudaStreamSynchronize(s));
@@ -420,6 +435,15 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     threads = std::max(64, (threads + 31) / 32 * 32);
     const long long gelems = o.group_elems > 0 ? o.group_elems : 262144;
 
+    // The panel kernel takes the batch where every LP's slices fit its shared
+    // memory: half an SM's, two CTAs per SM, on as many CTAs per LP as that
+    // needs.  The kernel that updates the tableau every pivot is for the rest.
+    const int drop = o.zero_skip != 0;
+    bool panel = true;
+    for (int k = 0; k < count && panel; ++k)
+        panel = panel_smem(prec, m[k], n[k] + m[k] + 1, std::min(sms, kPanelMaxCtas),
+                           kPanelBatchK) <= kPanelBatchSmem;
+
     // shapes: CTAs per LP from its tableau size, strips of whole sectors
     std::vector<int> M(count), N(count), G(count), W(count), sv(count);
     std::vector<long long> P(count);
@@ -429,6 +453,15 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         N[k] = n[k] + m[k] + 1;
         P[k] = pitch_for(N[k]);
         sv[k] = sense ? sense[k] : 0;
+        if (panel) {
+            long long g = ((long long)M[k] * P[k] + gelems - 1) / gelems;
+            g = std::max<long long>(1, std::min<long long>(g, std::min(std::min(sms, kPanelMaxCtas), N[k])));
+            while (panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK) > kPanelBatchSmem) ++g;
+            G[k] = (int)g;
+            W[k] = 0;
+            smem_max = std::max(smem_max, panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK));
+            continue;
+        }
         const long long gmin = (P[k] + (long long)threads * vw - 1) / ((long long)threads * vw);
         long long g = ((long long)M[k] * P[k] + gelems - 1) / gelems;
         g = std::min<long long>(g, std::min<long long>(sms, P[k] / sector));
@@ -443,9 +476,11 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         smem_max = std::max(smem_max, sprow + scol + sr);
         sprow_max = std::max(sprow_max, sprow);
     }
+    if (panel) threads = kPanelThreads;
     const int use_smem = smem_max <= 200 * 1024 ? 1 : 0;
     const size_t smem = use_smem ? smem_max : sprow_max;
-    const int ctas = max_coresident_batch_ctas(prec, threads, smem, use_smem, sms);
+    const int ctas = panel ? max_coresident_panel_batch_ctas(prec, smem, sms)
+                           : max_coresident_batch_ctas(prec, threads, smem, use_smem, sms);
     const int max_group = *std::max_element(G.begin(), G.end());
     if (ctas < max_group)
         return bfail(LP_ERR_INVALID_ARG, "lp_solve_batch: %d co-resident CTAs, a group needs %d",
@@ -489,13 +524,18 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
                  o_len = take(3 * count * sizeof(long long)), o_dst = take(3 * count * sizeof(long long)),
                  o_desc = take(count * sizeof(LpDesc));
     const size_t meta_bytes = off;
-    size_t basis_total = 0, part_total = 0;
+    // (panel kernel: `part` is its workspace, and records follow the barrier
+    // words of all LPs)
+    size_t basis_total = 0, part_total = 0, rec_total = 0;
     for (int k = 0; k < count; ++k) {
         basis_total += up256((size_t)m[k] * sizeof(int));
-        part_total += up256(2 * (size_t)G[k] * sizeof(Cand));
+        part_total += up256(panel ? panel_workspace(prec, m[k], N[k], P[k], G[k], kPanelBatchK)
+                                  : 2 * (size_t)G[k] * sizeof(Cand));
+        if (panel) rec_total += 256 * (size_t)G[k];
     }
+    const size_t bar_bytes = (size_t)count * 512 + rec_total;
     const size_t o_stats = take(count * sizeof(InputStats)), o_queue = take(sizeof(unsigned)),
-                 o_obj = take(count * sizeof(double)), o_bar = take((size_t)count * 512),
+                 o_obj = take(count * sizeof(double)), o_bar = take(bar_bytes),
                  o_basis = take(basis_total), o_part = take(part_total),
                  o_xy = take(xy_total * sizeof(double)), o_inp = take(in_total * sizeof(double)),
                  o_scr = take(scr_total), o_T = take(t_total);
@@ -587,7 +627,7 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     B_TRY(cudaStreamSynchronize(s));
 
     LpDesc *h_desc = reinterpret_cast<LpDesc *>(H + o_desc);
-    size_t bo = 0, po = 0;
+    size_t bo = 0, po = 0, ro = 0;
     for (int k = 0; k < count; ++k) {
         const InputStats &st = h_stats[k];
         if (st.flags & 4)
@@ -609,7 +649,13 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
             const size_t sr = (size_t)(sv[k] == 0 && !fp32 ? M[k] : N[k]) * sizeof(double);
             d.scratch_stride = (long long)up256(scol + sr);
         }
-        d.part_sel = reinterpret_cast<Cand *>(D + o_part + po);
+        if (panel) {
+            d.panel = D + o_part + po;
+            d.recs = D + o_bar + (size_t)count * 512 + ro;
+            ro += 256 * (size_t)G[k];
+        } else {
+            d.part_sel = reinterpret_cast<Cand *>(D + o_part + po);
+        }
         d.bar = reinterpret_cast<unsigned *>(D + o_bar + (size_t)k * 512);
         d.err = reinterpret_cast<int *>(d.bar + 96);
         d.P = P[k];
@@ -628,11 +674,12 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         d.strip = W[k];
         h_desc[k] = d;
         bo += up256((size_t)m[k] * sizeof(int));
-        po += up256(2 * (size_t)G[k] * sizeof(Cand));
+        po += up256(panel ? panel_workspace(prec, m[k], N[k], P[k], G[k], kPanelBatchK)
+                          : 2 * (size_t)G[k] * sizeof(Cand));
     }
     LpDesc *d_desc = reinterpret_cast<LpDesc *>(D + o_desc);
     B_TRY(cudaMemcpyAsync(d_desc, h_desc, count * sizeof(LpDesc), cudaMemcpyHostToDevice, s));
-    B_TRY(cudaMemsetAsync(D + o_bar, 0, (size_t)count * 512, s));
+    B_TRY(cudaMemsetAsync(D + o_bar, 0, bar_bytes, s));
     B_TRY(cudaMemsetAsync(D + o_queue, 0, sizeof(unsigned), s));
     if (fp32)
         batch_build_kernel<float><<<dim3(16, count), 256, 0, s>>>(
@@ -669,6 +716,9 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         f.smem = smem;
         f.use_smem = use_smem;
         f.sms = sms;
+        f.panel = panel;
+        f.drop = drop;
+        f.bar_bytes = bar_bytes;
         f.opt = &o;
         f.s = s;
         lp_status *fin = nullptr;
@@ -703,9 +753,14 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     B_TRY(cudaEventCreate(&e0));
     B_TRY(cudaEventCreate(&e1));
     B_TRY(cudaEventRecord(e0, s));
-    B_TRY(launch_batch(prec, d_desc, reinterpret_cast<const int2 *>(D + o_items), (int)items.size(),
-                       reinterpret_cast<unsigned *>(D + o_queue), ctas, threads, smem, use_smem,
-                       o.spin_timeout_cycles, o.max_iters, s));
+    if (panel)
+        B_TRY(launch_panel_batch(prec, d_desc, reinterpret_cast<const int2 *>(D + o_items),
+                                 (int)items.size(), reinterpret_cast<unsigned *>(D + o_queue), ctas,
+                                 smem, o.spin_timeout_cycles, o.max_iters, drop, s));
+    else
+        B_TRY(launch_batch(prec, d_desc, reinterpret_cast<const int2 *>(D + o_items),
+                           (int)items.size(), reinterpret_cast<unsigned *>(D + o_queue), ctas,
+                           threads, smem, use_smem, o.spin_timeout_cycles, o.max_iters, s));
     B_TRY(cudaEventRecord(e1, s));
     batch_extract_kernel<double><<<count, 256, 0, s>>>(ba, D + o_T,
                                                        reinterpret_cast<int *const *>(D + o_bptr),

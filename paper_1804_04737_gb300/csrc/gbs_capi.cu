@@ -393,10 +393,11 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     // updated there, and a CTA's few rows split unevenly (512 x 4096: 11.0 us
     // per pivot against 10.8).
     const int pdrop = h->opt.zero_skip == 2 || (h->opt.zero_skip == 1 && 4ll * m >= n);
-    const size_t pws = panel_workspace(h->prec, m, P);
+    const PivotShape psh = choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, (int)sense, pdrop);
+    const size_t pws = panel_workspace(h->prec, m, N, P, psh.ctas, kPanelK);
     bool panel = h->opt.pipeline == 1 &&
                  (4ll * m >= n || (long long)M * P < (1ll << 20)) && (pws <= (64ull << 20) || 2 * pws <= tbytes) &&
-                 choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, (int)sense, pdrop).pipe == 4;
+                 psh.pipe == 4;
     if (panel && h->region) {
         // (what the buffers below take besides the inputs, with slack)
         const size_t need = tbytes + pws + (size_t)(m + n) * 16 +
@@ -551,6 +552,7 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     d.T2 = have_t2 ? h->dT2 : nullptr;
     d.colx = h->dcolx;
     d.panel = h->dpanel;
+    d.recs = h->dbar + kBarWords;
     d.abort = h->opt.time_limit_s > 0.0 ? h->dabort : nullptr;
     d.work = reinterpret_cast<unsigned long long *>(h->dbar + kBarWords + kPanelRecWords);
     CUDA_TRY(h, cudaMemsetAsync(d.work, 0, 2 * sizeof(unsigned long long), s));

@@ -76,8 +76,10 @@ struct LpDesc {
     // nonzero when a constraint row may hold a -0 (from the data, Phase I,
     // FP32 mode, or a -0 an update produced): no vector is left in place
     int negz;
-    // panel kernel: its pending columns and rows (panel_workspace bytes)
-    void *panel;
+    // panel kernel: its pending columns and rows (panel_workspace bytes), and
+    // its records (2 exchanges x CTAs, a 128-byte line each; zeroed before a
+    // launch)
+    void *panel, *recs;
 };
 
 // Launch shape of the persistent pivot kernel for one LP.
@@ -110,7 +112,7 @@ constexpr int kBarWords = 256;
 // The panel kernel (gbs_panel.cu): pivots pending at most, CTA size, and CTAs
 // at most.  Its two record exchanges (a 128-byte line per CTA and exchange) follow
 // the synchronisation block and are zeroed with it before each launch.
-constexpr int kPanelK = 16;
+constexpr int kPanelK = 16, kPanelBatchK = 8;
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxCtas = 192;
 constexpr int kPanelRecWords = 2 * kPanelMaxCtas * 32;
@@ -165,9 +167,15 @@ cudaError_t launch_pivot_pipe(int prec, LpDesc *d_desc, const PivotShape &sh,
 // The panel kernel's shape (pipe == 0: its shared memory does not fit), its
 // workspace bytes and its launch (gbs_panel.cu).
 PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop);
-size_t panel_workspace(int prec, int m, long long P);
+size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K);
+size_t panel_smem(int prec, int m, int N, int G, int K);
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s);
+// The same over a batch's work items, panels of kPanelBatchK.
+cudaError_t launch_panel_batch(int prec, LpDesc *descs, const int2 *items, int nitems,
+                               unsigned *queue, int ctas, size_t smem, long long spin_limit,
+                               long long budget, int drop, cudaStream_t s);
+int max_coresident_panel_batch_ctas(int prec, size_t smem, int sms);
 cudaError_t launch_extract(int prec, const LpDesc *d_desc, const void *T, const int *basis,
                            int m, int n, long long P, int sense, double *x, double *y,
                            double *obj, cudaStream_t s);

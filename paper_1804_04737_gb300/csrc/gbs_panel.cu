@@ -257,11 +257,10 @@ __device__ __forceinline__ int min_lane(unsigned long long vk, int key) {
 // Pending pivots of one row or column entry lie side by side in shared memory,
 // kStride apart from the next entry's, so that a lane fetches all of its own
 // with 16-byte loads at constant offsets and 8 lanes' loads cover the banks.
-template <typename T>
-constexpr int kStride = sizeof(T) == 8 ? kPanelK + 2 : kPanelK + 4;
+__host__ __device__ constexpr int entry_stride(int esz, int K) { return esz == 8 ? K + 2 : K + 4; }
 
 // v <- fma(-c[t], p[t], v) for t in [0, k), in order (c, p: shared memory, at
-// least kStride entries).  A loop, with the next entries fetched ahead: the
+// least entry_stride).  A loop, with the next entries fetched ahead: the
 // fmas' latency is its only cost (unrolled and predicated, all 16 ran).
 template <typename T>
 __device__ __forceinline__ T fma_chain(T v, int k, const T *c, const T *p) {
@@ -291,9 +290,9 @@ struct PanelLayout {
     size_t zs, prs, cs, rh, bas, lastp, rowz, bb, stay, list, total;
 };
 
-__host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz, int vw) {
+__host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz, int vw, int K) {
     PanelLayout L;
-    const int stride = esz == 8 ? kStride<double> : kStride<float>;
+    const int stride = entry_stride(esz, K);
     L.R = (m + G - 1) / G + 1;  // slices differ by at most one row
     L.W = (N + G - 1) / G + 1;
     L.nvec = (N + vw - 1) / vw;
@@ -337,17 +336,18 @@ constexpr unsigned kFlagAll = 1u << 31;   // this panel gets every column
 constexpr unsigned kFlagZero = 1u << 30;  // the ratio rounds to zero
 constexpr unsigned kFlagWide = 1u << 29;  // a ratio key out of range
 
-template <typename T, bool DUAL>
-__global__ void __launch_bounds__(kPanelThreads, 1)
-    panel_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
-                 unsigned nonce) {
+// One LP on a group of G co-resident CTAs, this one its g-th, with panels of up
+// to K pivots.
+template <typename T, bool DUAL, int K>
+__device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g,
+                                            long long spin_limit, long long budget, int drop,
+                                            unsigned nonce, unsigned char *smem_raw) {
     typedef typename Vec<T>::type V;
     typedef typename DivisorOf<T>::type Divisor;
     constexpr int VW = Vec<T>::W;
-    constexpr int K = kPanelK, B = kPanelThreads, nw = kWarps, KS = kStride<T>;
+    constexpr int B = kPanelThreads, nw = kWarps, KS = entry_stride(sizeof(T), K);
     constexpr int RS = sizeof(T) == 8 ? 4 : 8;  // rows of a panel step in flight per warp
     constexpr unsigned kAll = 0xffffffffu;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Slot s_loc[nw], s_ex1[kPollWarps], s_ex2[kPollWarps], s_ex3[kPollWarps];
     __shared__ __align__(16) T s_at[nw][KS];  // a warp's pending entries at one row or column
     __shared__ int s_flag, s_fail[2], s_nflag, s_task, s_scan[nw];
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     __shared__ ulonglong2 s_rec[2];
     __shared__ unsigned long long s_aux[2][2][4];
 
-    const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x;
+    const int tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
     T *const Tab = reinterpret_cast<T *>(d->T);
     const long long P = d->P;
@@ -363,15 +363,16 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     const long long Mp = tag_pitch(m), Np = tag_pitch(N);
     // pending columns (K x Mp) and rows (K x Np) and the records' further values
     // (by pivot parity, 2 exchanges x G x 4) as 16-byte values with the tag of their pivot, for
-    // single entries; and the rows plain, for the panels
+    // single entries (with one CTA they are all in its shared memory); and the
+    // rows plain, for the panels
     ulonglong2 *const CT = reinterpret_cast<ulonglong2 *>(d->panel);
-    ulonglong2 *const PT = CT + (long long)K * Mp;
-    ulonglong2 *const AX = PT + (long long)K * Np;
-    T *const PR = reinterpret_cast<T *>(AX + 16 * kPanelMaxCtas);
-    ulonglong2 *const recs = reinterpret_cast<ulonglong2 *>(d->bar + kBarWords);
+    ulonglong2 *const PT = CT + (G > 1 ? K * Mp : 0);
+    ulonglong2 *const AX = PT + (G > 1 ? K * Np : 0);
+    T *const PR = reinterpret_cast<T *>(AX + (G > 1 ? 16 * G : 0));
+    ulonglong2 *const recs = reinterpret_cast<ulonglong2 *>(d->recs);
     int *const err = d->err;
 
-    const PanelLayout L = panel_layout(m, N, G, sizeof(T), VW);
+    const PanelLayout L = panel_layout(m, N, G, sizeof(T), VW, K);
     T *const zs = reinterpret_cast<T *>(smem_raw + L.zs);
     T *const prs = reinterpret_cast<T *>(smem_raw + L.prs);
     T *const cs = reinterpret_cast<T *>(smem_raw + L.cs);
@@ -630,7 +631,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     // parity: they are read up to the next selection, and the next but one's
     // records come only after that.
     auto further_at = [&](unsigned e, int which, int cta) {
-        return AX + 4 * (((int)(e & 1) * 2 + which) * kPanelMaxCtas + cta);
+        return AX + 4 * (((int)(e & 1) * 2 + which) * G + cta);
     };
     auto set_further = [&](int which, int i, unsigned long long v) {
         if (G == 1) s_aux[epoch & 1][which][i] = v;
@@ -640,7 +641,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     auto publish = [&](int which, unsigned long long x, int idx, unsigned flags) {
         const unsigned ix = (unsigned)(idx + 1) | flags;
         if (G == 1) s_rec[which] = make_ulonglong2(x, ix);
-        else st_half(recs + (which * kPanelMaxCtas + g) * kRec, x, ix, epoch);
+        else st_half(recs + (which * G + g) * kRec, x, ix, epoch);
     };
     // One round trip for what a warp needs of this pivot: pending entries
     // (lane t < k: pend + t * step, or own[t] where there is one CTA) into its
@@ -691,7 +692,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
         const int id = (which != 0) == DUAL ? 3 : 4;
         group_sync(id, id == 3 ? gate3 : gate4);
         const int e0 = (wid - kPollFirst) * 32 + lane;
-        const ulonglong2 *rec = recs + which * kPanelMaxCtas * kRec;
+        const ulonglong2 *rec = recs + which * G * kRec;
         const long long t0 = clock64();
         for (int spin = 0;; ++spin) {
             bool ok = true;
@@ -1347,41 +1348,88 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     }
 }
 
+template <typename T, bool DUAL>
+__global__ void __launch_bounds__(kPanelThreads, 1)
+    panel_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
+                 unsigned nonce) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    panel_solve<T, DUAL, kPanelK>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce, smem_raw);
+}
+
+// Many LPs in one launch.  items[] lists (lp, rank) pairs, the ranks of one LP
+// consecutive, largest LPs first; CTAs pop items in order from *queue, and the
+// d->group CTAs that pop the ranks of one LP solve it together.  A group waits
+// only on CTAs that hold earlier items, whose groups are complete, so every
+// group forms (the launch has at least max(group) co-resident CTAs).  Two CTAs
+// per SM (128 registers a thread, panels of 8): one LP's selection chain
+// overlaps another's panels.
+template <typename T>
+__global__ void __launch_bounds__(kPanelThreads, 2)
+    panel_batch_kernel(LpDesc *__restrict__ descs, const int2 *__restrict__ items, int nitems,
+                       unsigned *queue, long long spin_limit, long long budget, int drop,
+                       unsigned nonce) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_item;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(queue, 1u);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= nitems) break;
+        const int2 w = items[it];
+        LpDesc *d = descs + w.x;
+        if (d->sense)
+            panel_solve<T, true, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
+                                               smem_raw);
+        else
+            panel_solve<T, false, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
+                                                smem_raw);
+    }
+}
+
+// Tags of different launches differ, whichever handle's memory they meet.
+unsigned next_nonce() {
+    static std::atomic<unsigned> launches{0};
+    return ++launches;
+}
+
 }  // namespace
 
 PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop) {
     PivotShape sh;
     const int m = M - 1;
-    const int esz = prec == PREC_FP64 ? 8 : 4, vw = prec == PREC_FP64 ? 2 : 4;
     // Default grid: every SM, on small LPs one CTA per two rows or 32 columns,
     // whichever gives more (one row per CTA measured no faster: 64^2 6.7 us per
     // pivot on 16 to 152 CTAs, 256^2 7.2 on 114 and on 152).
     int G = ctas > 0 ? ctas : std::max((m + 1) / 2, (N + 31) / 32);
     G = std::min(G, std::min(sms, kPanelMaxCtas));
     G = std::max(1, std::min(G, N));
-    const PanelLayout L = panel_layout(m, N, G, esz, vw);
+    const size_t smem = panel_smem(prec, m, N, G, kPanelK);
     sh.ctas = G;
     sh.threads = kPanelThreads;
     sh.dual = dual;
     sh.drop = drop;
     sh.use_smem = 1;
-    sh.smem_bytes = L.total;
-    sh.pipe = L.total <= kMaxDynSmem ? 4 : 0;
+    sh.smem_bytes = smem;
+    sh.pipe = smem <= kMaxDynSmem ? 4 : 0;
     return sh;
 }
 
-size_t panel_workspace(int prec, int m, long long P) {
+size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K) {
     const size_t esz = prec == PREC_FP64 ? 8 : 4;
-    // (the pitch is at least n + m + 1)
-    return (size_t)kPanelK * ((size_t)(tag_pitch(m) + tag_pitch(P)) * 16 + (size_t)P * esz) + 256 * kPanelMaxCtas;
+    const size_t tagged =
+        G > 1 ? (size_t)K * (size_t)(tag_pitch(m) + tag_pitch(N)) * 16 + 256 * (size_t)G : 0;
+    return tagged + (size_t)K * (size_t)P * esz;
+}
+
+size_t panel_smem(int prec, int m, int N, int G, int K) {
+    return panel_layout(m, N, G, prec == PREC_FP64 ? 8 : 4, prec == PREC_FP64 ? 2 : 4, K).total;
 }
 
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s) {
     int drop = sh.drop;
-    // (tags of different launches differ, whichever handle's memory they meet)
-    static std::atomic<unsigned> launches{0};
-    unsigned nonce = ++launches;
+    unsigned nonce = next_nonce();
     void *args[] = {&d_desc, &spin_limit, &budget, &drop, &nonce};
     const void *fn = prec == PREC_FP64 ? (sh.dual ? (const void *)panel_kernel<double, true>
                                                   : (const void *)panel_kernel<double, false>)
@@ -1392,6 +1440,29 @@ cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long lo
     // A cooperative launch fails instead of running when the grid cannot be
     // co-resident, which the record exchanges need.
     return cudaLaunchCooperativeKernel(fn, dim3(sh.ctas), dim3(sh.threads), args, sh.smem_bytes, s);
+}
+
+cudaError_t launch_panel_batch(int prec, LpDesc *descs, const int2 *items, int nitems,
+                               unsigned *queue, int ctas, size_t smem, long long spin_limit,
+                               long long budget, int drop, cudaStream_t s) {
+    unsigned nonce = next_nonce();
+    void *args[] = {&descs, &items, &nitems, &queue, &spin_limit, &budget, &drop, &nonce};
+    const void *fn = prec == PREC_FP64 ? (const void *)panel_batch_kernel<double>
+                                       : (const void *)panel_batch_kernel<float>;
+    cudaError_t e = allow_dyn_smem(fn);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(kPanelThreads), args, smem, s);
+}
+
+int max_coresident_panel_batch_ctas(int prec, size_t smem, int sms) {
+    const void *fn = prec == PREC_FP64 ? (const void *)panel_batch_kernel<double>
+                                       : (const void *)panel_batch_kernel<float>;
+    allow_dyn_smem(fn);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPanelThreads, smem) !=
+        cudaSuccess)
+        return 0;
+    return per_sm * sms;
 }
 
 }  // namespace gbs
