@@ -17,15 +17,21 @@
 // groups in single-single (two-float) arithmetic and scales once in FP64, so
 // the FP64 pipe does a few operations per output, not one per group.
 //
-// Kernel (persistent, 192 threads, one CTA per SM): warp 0 issues the TMA
+// Kernel (persistent, 576 threads, one CTA per SM): warp 0 issues the TMA
 // loads (cp.async.bulk.tensor, 128-byte swizzle) of the A digit planes (a ring
-// of 4 stages of 128 x 64) and of all S B digit planes of a 64-column block
-// (two stages); warp 1 issues tcgen05.mma (M 128, N 64, K 16, bf16 in, FP32
+// of 3 stages of 128 x 64) and of all S B digit planes of a 64-column block
+// (three stages); warp 1 issues tcgen05.mma (M 128, N 64, K 16, bf16 in, FP32
 // accumulate) for the 28 digit pairs into S accumulators in tensor memory
-// (S x 64 of its 512 columns); warps 2-5 read the accumulators (tcgen05.ld) and
+// (S x 64 of its 512 columns); warps 2-17 read the accumulators (tcgen05.ld) and
 // write C.  Every wait is bounded: past the limit a role sets the error flag,
 // the others stop at their next wait, the loads in flight are waited for, and
 // tensor memory is freed before the CTA exits.
+//
+// Measured, 7858 x 16385 x 334 (13 of the 28 pairs not zero), clocks per tile of
+// 128 x 64: MMAs 15.8 K (50 each; reading their operands from shared memory
+// takes 48), the epilogue up to handing tensor memory back 5 K, waits for
+// operands 4.6 K (8.5 K with two B stages), 32.5 K in all (43 K before); the
+// epilogue's second half, 18 K, runs under the next tile's MMAs.
 //
 // The body refresh (FP32 mode, not in the paper; Sec. 2 Steps 4-5 produce the
 // tableau B^-1 [A I b] that it recomputes): with S the structural basic
@@ -62,14 +68,14 @@ constexpr int kOzS = 7;                 // digits per operand
 constexpr int kOzT = 7;                 // bits per digit
 constexpr int kOzBM = 128, kOzBN = 64, kOzBK = 64;
 constexpr int kOzChunkKB = 7;           // K blocks per exact group sum (448 terms)
-constexpr int kOzAStages = 4;
+constexpr int kOzAStages = 3, kOzBStages = 3;
 constexpr int kOzABytes = kOzBM * kOzBK * 2;            // 16 KB: one A digit plane block
 constexpr int kOzBBytes = kOzBN * kOzBK * 2;            // 8 KB: one B digit plane block
 constexpr int kOzBStageBytes = kOzS * kOzBBytes;        // 56 KB: all digit planes of a B block
 constexpr int kOzTmemCols = 512;                        // S x 64 = 448 used
 constexpr int kOzEpiWarps = 16;         // epilogue warps: four per tensor-memory lane quarter
 constexpr int kOzThreads = 64 + 32 * kOzEpiWarps;
-constexpr size_t kOzSmem = 1024 + 2 * kOzBStageBytes + kOzAStages * kOzABytes + 256;
+constexpr size_t kOzSmem = 1024 + kOzBStages * kOzBStageBytes + kOzAStages * kOzABytes + 256;
 
 static_assert(kOzS * kOzBN <= kOzTmemCols, "accumulators must fit tensor memory");
 static_assert(kOzT * kOzS == 49, "the digit extraction below assumes 49 bits");
@@ -101,9 +107,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // Bounded wait for the phase of the given parity; false when the limit ran out
 // or another CTA or role flagged an error.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *err, long long limit) {
+    // (the flag is in global memory: asked for at every try, its round trip made
+    // each wait of the loader and the MMA issuer hundreds of clocks late)
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*(volatile int *)err) return false;
+    for (int spin = 1; !mbar_try_wait(bar, parity); ++spin) {
+        if ((spin & 31) == 0 && *(volatile int *)err) return false;
         if (clock64() - t0 > limit) {
             atomicExch(err, 1);
             return false;
@@ -129,25 +137,27 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accum) {
+// Four K steps of 16 of one 128 x 64 x 64 product: each advances the operands'
+// descriptors by 32 bytes; the first overwrites D where accum is 0.
+__device__ __forceinline__ void tc_mma4(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accum) {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "{\n.reg .pred p, q;\n.reg .b64 a1, a2, a3, b1, b2, b3;\n"
+        "setp.ne.b32 p, %4, 0;\nsetp.eq.b32 q, 0, 0;\n"
+        "add.s64 a1, %1, 2;\nadd.s64 a2, %1, 4;\nadd.s64 a3, %1, 6;\n"
+        "add.s64 b1, %2, 2;\nadd.s64 b2, %2, 4;\nadd.s64 b3, %2, 6;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, q;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, q;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, q;\n}\n" ::"r"(dtmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-        "%12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, "
-        "%30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-          "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-          "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
+// True in one lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
@@ -158,14 +168,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                   "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
 __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Keeps the uses of loaded accumulators behind the wait before this.
+__device__ __forceinline__ void tmem_use(uint32_t (&r)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) asm volatile("" : "+r"(r[j]));
 }
 
 // Shared-memory matrix descriptor of a K-major operand block in the 128-byte
@@ -472,15 +482,15 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     __shared__ int s_colexp[kOzBN], s_brow[kOzBN];
     const uint32_t raw = su32(oz_smem);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t sB = base;                                  // [2][S][64][128 B]
-    const uint32_t sA = base + 2 * kOzBStageBytes;             // [4][128][128 B]
+    const uint32_t sB = base;                                  // [stages][S][64][128 B]
+    const uint32_t sA = base + kOzBStages * kOzBStageBytes;    // [stages][128][128 B]
     const uint32_t sBar = sA + kOzAStages * kOzABytes;         // barriers, 8 bytes each
     auto full_a = [&](int s) { return sBar + 8u * s; };
     auto empty_a = [&](int s) { return sBar + 8u * (kOzAStages + s); };
     auto full_b = [&](int s) { return sBar + 8u * (2 * kOzAStages + s); };
-    auto empty_b = [&](int s) { return sBar + 8u * (2 * kOzAStages + 2 + s); };
-    const uint32_t tmem_full = sBar + 8u * (2 * kOzAStages + 4);
-    const uint32_t tmem_empty = sBar + 8u * (2 * kOzAStages + 5);
+    auto empty_b = [&](int s) { return sBar + 8u * (2 * kOzAStages + kOzBStages + s); };
+    const uint32_t tmem_full = sBar + 8u * (2 * kOzAStages + 2 * kOzBStages);
+    const uint32_t tmem_empty = tmem_full + 8u;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -488,7 +498,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             mbar_init(full_a(s), 1);
             mbar_init(empty_a(s), 1);
         }
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < kOzBStages; ++s) {
             mbar_init(full_b(s), 1);
             mbar_init(empty_b(s), 1);
         }
@@ -532,7 +542,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                         if ((mb >> q) & 1)
                             tma_load_2d(sB + bs * kOzBStageBytes + q * kOzBBytes, &tmB, kb * kOzBK,
                                         q * p.Np + n0, full_b(bs));
-                    if (++bs == 2) {
+                    if (++bs == kOzBStages) {
                         bs = 0;
                         bph ^= 1u;
                     }
@@ -556,7 +566,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     const long long t0 = clock64();
                     while (!mbar_try_wait(full_a(s), ((s < as) ? aph : aph ^ 1u)) && clock64() - t0 < lim) {}
                 }
-                for (int s = 0; s < 2; ++s) {
+                for (int s = 0; s < kOzBStages; ++s) {
                     const long long t0 = clock64();
                     while (!mbar_try_wait(full_b(s), ((s < bs) ? bph : bph ^ 1u)) && clock64() - t0 < lim) {}
                 }
@@ -564,73 +574,89 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         }
     } else if (warp == 1) {
         // ---- MMA issuer ----
-        if (lane == 0) {
-            int as = 0, bs = 0;
-            uint32_t aph = 0, bph = 0, use = 0;
-            unsigned long long nmma = 0;  // MMA instructions issued
-            bool ok = true;
-            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-                const int ma = p.amask[(t % nmb)], mb = p.bmask[(t / nmb)];
-                for (int c = 0; c < nch && ok; ++c) {
-                    // the epilogue has drained the accumulators of the last use
-                    if (!(ok = mbar_wait(tmem_empty, (use & 1u) ^ 1u, p.err, lim))) break;
-                    tc_fence_after();
-                    const int kb0 = c * kOzChunkKB, kb1 = min(nkb, kb0 + kOzChunkKB);
-                    uint32_t inited = 0u;  // accumulator groups written in this chunk
-                    for (int kb = kb0; kb < kb1 && ok; ++kb) {
-                        // (TMA-written shared memory is read by the MMAs, both
-                        // async-proxy operations: the barrier wait orders them)
-                        if (!(ok = mbar_wait(full_b(bs), bph, p.err, lim))) break;
-                        // descriptors: B digit plane q of this stage is 8 KB
-                        // (512 descriptor units) after plane 0; each K step of 16
-                        // elements advances a descriptor by 32 bytes (2 units)
-                        const uint64_t bd0 = sw128_desc(sB + bs * kOzBStageBytes);
-                        for (int pp = 0; pp < kOzS; ++pp) {
-                            if (!((ma >> pp) & 1)) continue;
-                            if (!(ok = mbar_wait(full_a(as), aph, p.err, lim))) break;
-                            const uint64_t ad = sw128_desc(sA + as * kOzABytes);
-#pragma unroll
-                            for (int q = 0; q < kOzS; ++q) {
-                                if (q < kOzS - pp && ((mb >> q) & 1)) {
-                                    // the first product into a group of this chunk
-                                    // overwrites it
-                                    const uint32_t acc0 = (inited >> (pp + q)) & 1u;
-                                    inited |= 1u << (pp + q);
-                                    const uint32_t d = tmem + (uint32_t)((pp + q) * kOzBN);
-                                    const uint64_t bd = bd0 + (uint64_t)(q * (kOzBBytes >> 4));
-                                    tc_mma(d, ad, bd, kOzIdesc, acc0);
-                                    tc_mma(d, ad + 2, bd + 2, kOzIdesc, 1u);
-                                    tc_mma(d, ad + 4, bd + 4, kOzIdesc, 1u);
-                                    tc_mma(d, ad + 6, bd + 6, kOzIdesc, 1u);
-                                    nmma += 4;
-                                }
-                            }
-                            tc_commit(empty_a(as));  // the stage frees when these MMAs complete
-                            if (++as == kOzAStages) {
-                                as = 0;
-                                aph ^= 1u;
-                            }
-                        }
+        // The whole warp runs the loops, so that descriptors and addresses stay
+        // in uniform registers; one elected lane issues.  (With lane 0 alone in
+        // the loops each MMA took 103 clocks to issue, most of them moving its
+        // operands to uniform registers, against the 48 clocks its operands
+        // take to read.)
+        const bool leader = elect_one();
+        int as = 0, bs = 0;
+        uint32_t aph = 0, bph = 0, use = 0;
+        unsigned long long nmma = 0;  // MMA instructions issued
+        bool ok = true;
+        // (the next tile's masks are asked for a tile ahead)
+        int ma_n = p.amask[min((int)blockIdx.x, tiles - 1) % nmb],
+            mb_n = p.bmask[min((int)blockIdx.x, tiles - 1) / nmb];
+        for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+            const int ma = __shfl_sync(0xffffffffu, ma_n, 0), mb = __shfl_sync(0xffffffffu, mb_n, 0);
+            const int tn = min(t + (int)gridDim.x, tiles - 1);
+            ma_n = p.amask[tn % nmb];
+            mb_n = p.bmask[tn / nmb];
+            for (int c = 0; c < nch && ok; ++c) {
+                // the epilogue has drained the accumulators of the last use
+                ok = __all_sync(0xffffffffu, mbar_wait(tmem_empty, (use & 1u) ^ 1u, p.err, lim));
+                if (!ok) break;
+                tc_fence_after();
+                const int kb0 = c * kOzChunkKB, kb1 = min(nkb, kb0 + kOzChunkKB);
+                uint32_t inited = 0u;  // accumulator groups written in this chunk
+                for (int kb = kb0; kb < kb1 && ok; ++kb) {
+                    // (TMA-written shared memory is read by the MMAs, both
+                    // async-proxy operations: the barrier wait orders them)
+                    ok = __all_sync(0xffffffffu, mbar_wait(full_b(bs), bph, p.err, lim));
+                    if (!ok) break;
+                    // descriptors: B digit plane q of this stage is 8 KB
+                    // (512 descriptor units) after plane 0; each K step of 16
+                    // elements advances a descriptor by 32 bytes (2 units)
+                    const uint64_t bd0 = sw128_desc(sB + bs * kOzBStageBytes);
+                    for (int pp = 0; pp < kOzS; ++pp) {
+                        if (!((ma >> pp) & 1)) continue;
+                        ok = __all_sync(0xffffffffu, mbar_wait(full_a(as), aph, p.err, lim));
                         if (!ok) break;
-                        tc_commit(empty_b(bs));
-                        if (++bs == 2) {
-                            bs = 0;
-                            bph ^= 1u;
+                        const uint64_t ad = sw128_desc(sA + as * kOzABytes);
+                        const uint32_t d0 = tmem + (uint32_t)(pp * kOzBN);
+                        const uint32_t qm = (uint32_t)mb & ((1u << (kOzS - pp)) - 1u);
+                        // the first product into a group of this chunk overwrites it
+                        const uint32_t acc = inited >> pp;
+                        inited |= qm << pp;
+                        nmma += 4 * __popc(qm);
+                        if (leader) {
+#pragma unroll
+                            for (int q = 0; q < kOzS; ++q)
+                                if ((qm >> q) & 1u)
+                                    tc_mma4(d0 + (uint32_t)(q * kOzBN), ad,
+                                            bd0 + (uint64_t)(q * (kOzBBytes >> 4)), kOzIdesc,
+                                            (acc >> q) & 1u);
+                            tc_commit(empty_a(as));  // the stage frees when these MMAs complete
+                        }
+                        __syncwarp();
+                        if (++as == kOzAStages) {
+                            as = 0;
+                            aph ^= 1u;
                         }
                     }
                     if (!ok) break;
-                    tc_commit(tmem_full);
-                    ++use;
+                    if (leader) tc_commit(empty_b(bs));
+                    __syncwarp();
+                    if (++bs == kOzBStages) {
+                        bs = 0;
+                        bph ^= 1u;
+                    }
                 }
+                if (!ok) break;
+                if (leader) tc_commit(tmem_full);
+                __syncwarp();
+                ++use;
             }
-            if (p.mmas) atomicAdd(p.mmas, nmma);
-            // every MMA issued is complete before tensor memory is freed
-            // (a commit arrives after all of them)
-            if (!ok) {
-                tc_commit(tmem_full);
-                const long long t0 = clock64();
-                while (!mbar_try_wait(tmem_full, use & 1u) && clock64() - t0 < lim) {}
-            }
+        }
+        if (lane == 0 && p.mmas) atomicAdd(p.mmas, nmma);
+        // every MMA issued is complete before tensor memory is freed
+        // (a commit arrives after all of them)
+        if (!ok) {
+            if (leader) tc_commit(tmem_full);
+            __syncwarp();
+            const long long t0 = clock64();
+            while (!mbar_try_wait(tmem_full, use & 1u) && clock64() - t0 < lim) {}
+            __syncwarp();
         }
     } else {
         // ---- epilogue: warps 2..17, TMEM lanes 32 (warp % 4) .. + 31; warps
@@ -641,124 +667,136 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
             const int m0 = (t % nmb) * kOzBM, n0 = (t / nmb) * kOzBN;
             const int r = m0 + lg * 32 + lane;  // this thread's output row
+            // the tile's column exponents (and basic rows) in shared memory,
+            // read by every lane at once (a broadcast), and the accumulator
+            // groups the MMA issuer writes, while its MMAs run
+            named_bar(1, 32 * kOzEpiWarps);  // the previous tile's reads of them are done
+            if (et < kOzBN) {
+                const int col = n0 + et;
+                s_colexp[et] = col < p.N ? p.colexp[col] : kNoExp;
+                if (p.mode == 1) s_brow[et] = col < p.N - 1 ? p.basic_row[col] : -1;
+            }
+            const int Er = r < p.M ? p.rowexp[r] : kNoExp;
+            uint32_t gm = 0u;
+            {
+                const int ma = p.amask[m0 / kOzBM], mb = p.bmask[n0 / kOzBN];
+                for (int pa = 0; pa < kOzS; ++pa)
+                    if ((ma >> pa) & 1) gm |= ((uint32_t)mb & ((1u << (kOzS - pa)) - 1u)) << pa;
+            }
+            // mode 1: this row's place in the tableau and its constraint, and its
+            // original entries at the warp's first 8 columns (the others follow
+            // once the accumulators are read)
+            int ti = 0, kr = 0;
+            const double *arow = p.Aorig;
+            double av[8];
+            auto orig = [&](double (&x)[8], int j0) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = j0 + j < p.n ? __ldg(arow + j0 + j) : 0.0;
+            };
+            if (p.mode == 1 && r < p.M) {
+                ti = p.rowmap[r];
+                kr = p.rowk[r];
+                arow += (long long)kr * p.n;
+                orig(av, n0 + hsel * 16);
+            }
             for (int c = 0; c < nch && ok; ++c) {
                 // all the epilogue warps leave together or go on together
-                // (this barrier also follows the previous tile's reads of
-                // the shared column data)
                 ok = named_bar_and(1, 32 * kOzEpiWarps, mbar_wait(tmem_full, use & 1u, p.err, lim));
                 if (!ok) break;
                 tc_fence_after();
-                const int Er = r < p.M ? p.rowexp[r] : kNoExp;
-                // the tile's column exponents (and basic rows) in shared
-                // memory, read by every lane at once (a broadcast)
-                if (et < kOzBN) {
-                    const int col = n0 + et;
-                    s_colexp[et] = col < p.N ? p.colexp[col] : kNoExp;
-                    if (p.mode == 1) s_brow[et] = col < p.N - 1 ? p.basic_row[col] : -1;
-                }
-                named_bar(1, 32 * kOzEpiWarps);
                 const uint32_t tbase = tmem + ((uint32_t)(lg * 32) << 16);
-                // the accumulator groups the MMA issuer wrote for this tile
-                uint32_t gm = 0u;
                 {
-                    const int ma = p.amask[m0 / kOzBM], mb = p.bmask[n0 / kOzBN];
-                    for (int pa = 0; pa < kOzS; ++pa)
-                        if ((ma >> pa) & 1)
-                            for (int qb = 0; qb < kOzS - pa; ++qb)
-                                if ((mb >> qb) & 1) gm |= 1u << (pa + qb);
-                }
-                {
-                    // the warp's 16 columns in two blocks of 8 (few enough
-                    // registers for four epilogue warps per lane quarter)
-                    int ti = 0, kr = 0;  // mode 1: this row's place in the tableau, its constraint
-                    if (p.mode == 1 && r < p.M) {
-                        ti = p.rowmap[r];
-                        kr = p.rowk[r];
-                    }
-                    const double *arow = p.Aorig + (long long)kr * p.n;
-#pragma unroll 1
-                    for (int sb = 0; sb < 2; ++sb) {
-                        const int cb = hsel * 16 + sb * 8;  // the block's first column in the tile
-                        const int j0 = n0 + cb;
-                        // mode 1: the row's original entries at the block's
-                        // columns, read before the accumulators so that their
-                        // latency overlaps the reads of tensor memory
-                        double av[8];
-                        if (p.mode == 1 && r < p.M) {
+                    // The warp's 16 columns: every group of accumulators is read and
+                    // combined first (the next group's read in flight), and tensor
+                    // memory handed back to the MMAs of the next tile; the scaling
+                    // in FP64, the reads of A's rows and the stores run under them.
+                    // (Handing it back after the first 8 columns' stores left the
+                    // tensor cores idle for half of each tile: 2.45 ms for the
+                    // 7858 x 16385 x 334 product, with the MMA issue below 1.81.)
+                    const int cb = hsel * 16;
+                    const int j0 = n0 + cb;
+                    float hi[16], lo[16];
+                    uint32_t v[2][16];
+                    tmem_ld16(tbase + (uint32_t)cb, v[0]);
+                    tmem_ld_wait();
+                    tmem_use(v[0]);
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) av[j] = j0 + j < p.n ? __ldg(arow + j0 + j) : 0.0;
+                    for (int g = 0; g < kOzS; ++g) {
+                        if (g + 1 < kOzS)
+                            tmem_ld16(tbase + (uint32_t)((g + 1) * kOzBN + cb), v[(g + 1) & 1]);
+                        const float sc = pow2f(-kOzT * g);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            // (a group no digit pair wrote holds stale columns: zero)
+                            const float x = ((gm >> g) & 1u)
+                                                ? __fmul_rn(__uint_as_float(v[g & 1][j]), sc)  // exact
+                                                : 0.0f;
+                            if (g == 0) {
+                                hi[j] = x;
+                                lo[j] = 0.0f;
+                            } else {
+                                float s, e;
+                                two_sum(hi[j], x, s, e);
+                                hi[j] = s;
+                                lo[j] = __fadd_rn(lo[j], e);
+                            }
                         }
-                        float hi[8], lo[8];
-#pragma unroll
-                        for (int g = 0; g < kOzS; ++g) {
-                            uint32_t v[8];
-                            tmem_ld8(tbase + (uint32_t)(g * kOzBN + cb), v);
+                        if (g + 1 < kOzS) {
                             tmem_ld_wait();
-                            const float sc = pow2f(-kOzT * g);
+                            tmem_use(v[(g + 1) & 1]);
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tmem_empty);
+                    // Each thread writes its own row's results (the row its
+                    // tensor-memory lane holds): one contiguous row segment per
+                    // thread, read (C, or the original row of A) and written with
+                    // independent accesses, no shared-memory transposition.
+                    if (p.mode == 0) {
+                        if (r < p.M) {
+                            double *crow = p.C + (long long)r * p.ldc + j0;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                // (a group no digit pair wrote holds stale columns: zero)
-                                const float x = ((gm >> g) & 1u)
-                                                    ? __fmul_rn(__uint_as_float(v[j]), sc)  // exact
-                                                    : 0.0f;
-                                if (g == 0) {
-                                    hi[j] = x;
-                                    lo[j] = 0.0f;
-                                } else {
-                                    float s, e;
-                                    two_sum(hi[j], x, s, e);
-                                    hi[j] = s;
-                                    lo[j] = __fadd_rn(lo[j], e);
-                                }
+                            for (int j = 0; j < 16; ++j) {
+                                const int Fc = s_colexp[cb + j];
+                                double v = 0.0;
+                                // scale 2^(Er - 1022 + Fc - 1022 - 14)
+                                if (Er != kNoExp && Fc != kNoExp) v = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
+                                if (j0 + j < p.N) crow[j] = c == 0 ? v : crow[j] + v;
                             }
                         }
-                        if (sb == 1) {
-                            // this warp's accumulators are in registers: once every
-                            // epilogue warp's are, the MMAs of the next tile may
-                            // start while the results are written
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(tmem_empty);
-                        }
-                        // Each thread writes its own row's results (the row its
-                        // tensor-memory lane holds): one contiguous row segment per
-                        // thread, read (C, or the original row of A) and written with
-                        // independent accesses, no shared-memory transposition.
-                        if (p.mode == 0) {
-                            if (r < p.M) {
-                                double *crow = p.C + (long long)r * p.ldc + j0;
+                    } else if (r < p.M) {
+                        const long long sgbit = p.sg < 0.0 ? (long long)kSign : 0ll;
+                        float *trow = p.T32 + (long long)ti * p.P;
+                        double aw[8];
+                        orig(aw, j0 + 8);
+                        auto refreshed = [&](int j, double aj) {
+                            const int col = j0 + j, br = s_brow[cb + j];
+                            if (br >= 0) return br == ti ? 1.0f : 0.0f;
+                            const int Fc = s_colexp[cb + j];
+                            double v = 0.0;
+                            if (Er != kNoExp && Fc != kNoExp)
+                                v = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
+                            // sg A_kj by its sign bit (no FP64 multiply)
+                            const double d = col < p.n ? __longlong_as_double(__double_as_longlong(aj) ^ sgbit)
+                                                       : (col - p.n == kr ? 1.0 : 0.0);
+                            return __double2float_rn(d - v);
+                        };
+                        // (the rhs column comes from the reinversion; the rows
+                        // are 128-byte aligned, the columns here 64)
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) {
-                                    const int Fc = s_colexp[cb + j];
-                                    double v = 0.0;
-                                    // scale 2^(Er - 1022 + Fc - 1022 - 14)
-                                    if (Er != kNoExp && Fc != kNoExp) v = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
-                                    if (j0 + j < p.N) crow[j] = c == 0 ? v : crow[j] + v;
-                                }
-                            }
-                        } else if (r < p.M) {
-                            const long long sgbit = p.sg < 0.0 ? (long long)kSign : 0ll;
-                            float *trow = p.T32 + (long long)ti * p.P;
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int col = j0 + j;
-                                // the rhs column comes from the reinversion
-                                if (col < p.N - 1) {
-                                    const int br = s_brow[cb + j];
-                                    float out;
-                                    if (br >= 0) {
-                                        out = br == ti ? 1.0f : 0.0f;
-                                    } else {
-                                        const int Fc = s_colexp[cb + j];
-                                        double v = 0.0;
-                                        if (Er != kNoExp && Fc != kNoExp) v = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
-                                        // sg A_kj by its sign bit (no FP64 multiply)
-                                        const double d = col < p.n ? __longlong_as_double(__double_as_longlong(av[j]) ^ sgbit)
-                                                                   : (col - p.n == kr ? 1.0 : 0.0);
-                                        out = __double2float_rn(d - v);
-                                    }
-                                    trow[col] = out;
-                                }
+                        for (int j = 0; j < 16; j += 4) {
+                            float4 o;
+                            o.x = refreshed(j, j < 8 ? av[j & 7] : aw[j & 7]);
+                            o.y = refreshed(j + 1, j < 8 ? av[(j & 7) + 1] : aw[(j & 7) + 1]);
+                            o.z = refreshed(j + 2, j < 8 ? av[(j & 7) + 2] : aw[(j & 7) + 2]);
+                            o.w = refreshed(j + 3, j < 8 ? av[(j & 7) + 3] : aw[(j & 7) + 3]);
+                            if (j0 + j + 3 < p.N - 1) {
+                                *reinterpret_cast<float4 *>(trow + j0 + j) = o;
+                            } else {
+                                if (j0 + j < p.N - 1) trow[j0 + j] = o.x;
+                                if (j0 + j + 1 < p.N - 1) trow[j0 + j + 1] = o.y;
+                                if (j0 + j + 2 < p.N - 1) trow[j0 + j + 2] = o.z;
                             }
                         }
                     }
