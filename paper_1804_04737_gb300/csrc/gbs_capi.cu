@@ -622,12 +622,31 @@ bool past_deadline(const lp_handle *h) {
     return h->opt.time_limit_s > 0.0 && std::chrono::steady_clock::now() >= h->deadline;
 }
 
+// A launch's shape with what is left of the wall-clock limit.
+PivotShape timed(const lp_handle *h, PivotShape sh) {
+    if (h->opt.time_limit_s > 0.0) {
+        const auto left = h->deadline - std::chrono::steady_clock::now();
+        sh.limit_ns = std::max<long long>(
+            1, std::chrono::duration_cast<std::chrono::nanoseconds>(left).count());
+    }
+    return sh;
+}
+
 // Wait for the handle's stream.  Under a wall-clock limit the host polls the
 // stream and, once the deadline has passed, raises the abort word, which
 // every pivot kernel reads once per pass: the kernel stops within a pass
 // with status LP_TIMEOUT and the wait ends.
 cudaError_t wait_stream(lp_handle *h) {
-    if (h->opt.time_limit_s <= 0.0) return cudaStreamSynchronize(h->stream);
+    if (h->opt.time_limit_s <= 0.0) {
+        // (a server's lanes give their cores up while they wait: the spinning
+        // wait kept a submitting thread off a busy host for milliseconds)
+        if (h->region) {
+            cudaError_t e;
+            while ((e = cudaStreamQuery(h->stream)) == cudaErrorNotReady) std::this_thread::yield();
+            return e;
+        }
+        return cudaStreamSynchronize(h->stream);
+    }
     bool raised = false;
     for (;;) {
         const cudaError_t e = cudaStreamQuery(h->stream);
@@ -739,6 +758,10 @@ lp_err refresh_body(lp_handle *h) {
         set_err(h, "reinversion: a wait of the body refresh ran out");
         return LP_ERR_CUDA;
     }
+    // the basic columns were written as exact unit vectors, +0 elsewhere
+    const int negz = 3;
+    CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, negz), &negz, sizeof negz,
+                                cudaMemcpyHostToDevice, s));
     return LP_OK;
 }
 
@@ -768,7 +791,8 @@ lp_err solve_fp32(lp_handle *h) {
                                     sizeof stride, cudaMemcpyHostToDevice, s));
         CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape_alt), s));
         CUDA_TRY(h, cudaEventRecord(h->ev0, s));
-        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, sh, h->opt.spin_timeout_cycles, budget, s));
+        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, sh), h->opt.spin_timeout_cycles, budget,
+                                 s));
         CUDA_TRY(h, cudaEventRecord(h->ev1, s));
         CUDA_TRY(h, cudaMemcpyAsync(h->pdesc, h->ddesc, sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(h, wait_stream(h));
@@ -873,8 +897,8 @@ lp_err lp_solve_async(lp_handle *h) {
         // host waits for its end to choose what follows.
         const long long before = h->pdesc->iters;
         CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
-        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, h->shape_alt, h->opt.spin_timeout_cycles,
-                                 budget, s));
+        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, h->shape_alt),
+                                 h->opt.spin_timeout_cycles, budget, s));
         CUDA_TRY(h, cudaMemcpyAsync(h->pdesc, h->ddesc, sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(h, wait_stream(h));
         adopt_tableau(h);
@@ -905,7 +929,8 @@ lp_err lp_solve_async(lp_handle *h) {
         }
     }
     CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
-    CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, h->shape, h->opt.spin_timeout_cycles, budget, s));
+    CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, h->shape), h->opt.spin_timeout_cycles,
+                             budget, s));
     CUDA_TRY(h, cudaEventRecord(h->ev1, s));
     CUDA_TRY(h, launch_extract(h->prec, h->ddesc, h->dT, h->dbasis, h->m, h->n, h->P, h->sense,
                                h->dx, h->dy, h->dobj, s));

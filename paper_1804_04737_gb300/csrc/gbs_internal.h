@@ -74,7 +74,8 @@ struct LpDesc {
     // passes; nullptr: not counted
     unsigned long long *work;
     // nonzero when a constraint row may hold a -0 (from the data, Phase I,
-    // FP32 mode, or a -0 an update produced): no vector is left in place
+    // FP32 mode, or a -0 an update produced): no vector is left in place; bit 1:
+    // the basic columns are known to be exact unit vectors with +0 elsewhere
     int negz;
     // panel kernel: its pending columns and rows (panel_workspace bytes), and
     // its records (2 exchanges x CTAs, a 128-byte line each; zeroed before a
@@ -96,6 +97,7 @@ struct PivotShape {
     int split = 0;                 // two pivots per pass, primal: first column of every CTA's second
                                    // run (0: one contiguous strip, every vector updated)
     int drop = 0;                  // panel kernel: leave out columns that stay basic
+    long long limit_ns = 0;        // panel kernel: wall-clock limit of a launch, 0 = none
     size_t smem_bytes = 0;         // dynamic shared memory per CTA
     long long scratch_stride = 0;  // global scratch bytes per CTA when !use_smem
 };

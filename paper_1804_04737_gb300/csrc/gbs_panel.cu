@@ -114,7 +114,13 @@ __device__ __forceinline__ bool not_finite(float x) {
     return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u;
 }
 
-// 16-byte record halves, written and read whole.
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// 16-byte values, written and read whole.
 __device__ __forceinline__ void st_half(ulonglong2 *p, unsigned long long a, unsigned lo,
                                         unsigned hi) {
     const unsigned long long b = ((unsigned long long)hi << 32) | lo;
@@ -341,12 +347,13 @@ constexpr unsigned kFlagWide = 1u << 29;  // a ratio key out of range
 template <typename T, bool DUAL, int K>
 __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g,
                                             long long spin_limit, long long budget, int drop,
-                                            unsigned nonce, unsigned char *smem_raw) {
+                                            unsigned nonce, long long limit_ns,
+                                            unsigned char *smem_raw) {
     typedef typename Vec<T>::type V;
     typedef typename DivisorOf<T>::type Divisor;
     constexpr int VW = Vec<T>::W;
     constexpr int B = kPanelThreads, nw = kWarps, KS = entry_stride(sizeof(T), K);
-    constexpr int RS = sizeof(T) == 8 ? 4 : 8;  // rows of a panel step in flight per warp
+    constexpr int RS = sizeof(T) == 8 || K < kPanelK ? 4 : 8;  // rows of a panel step per warp
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ Slot s_loc[nw], s_ex1[kPollWarps], s_ex2[kPollWarps], s_ex3[kPollWarps];
     __shared__ __align__(16) T s_at[nw][KS];  // a warp's pending entries at one row or column
@@ -405,8 +412,9 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         iters > 0x3fffffffffffffffll - budget ? 0x3fffffffffffffffll : iters + budget;
     int deg = d->deg;
     int status = ST_RUNNING;
-    const bool scan = drop && iters > 0 && (DUAL || d->negz);
+    const bool scan = drop && iters > 0 && (DUAL || d->negz) && !(d->negz & 2);
     const int *const abort_word = d->abort;
+    const unsigned long long t_start = limit_ns > 0 ? global_ns() : 0ull;
     const long long trace_cap = d->trace_cap;
 
     // ------------------------------------------------------------- start --
@@ -447,9 +455,16 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             for (int r = wid; r < R; r += nw) {
                 const T *row = Tab + (long long)(i0 + r) * P;
                 int bad = 0;
-                for (int j = lane; j < N; j += 32) {
-                    if (!(bb[j >> 5] >> (j & 31) & 1u) || j == bas[r]) continue;
-                    bad |= to_bits(lds(row + j)) != 0ull;
+                for (int j0 = 0; j0 < N; j0 += 256) {
+                    T x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = lds(row + min(j0 + 32 * u + lane, N - 1));
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int j = j0 + 32 * u + lane;
+                        bad |= j < N && (bb[(j0 >> 5) + u] >> lane & 1u) && j != bas[r] &&
+                               to_bits(x[u]) != 0ull;
+                    }
                 }
                 if (__any_sync(kAll, bad) && lane == 0) {
                     rowz[r] = 1;
@@ -469,12 +484,10 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     unsigned long long upd = 0, left = 0;  // vectors x pivots, for d->work
 
     // NR rows of one 16-byte vector column: kk pending pivots on each.
-    auto panel_rows = [&](auto nr_tag, V *at, int r, int kk, const V(&pr)[K], bool act) {
+    const long long pv = P / VW;
+    auto panel_rows = [&](auto nr_tag, V(&a)[decltype(nr_tag)::value], V *at, int r, int kk,
+                          const V(&pr)[K], bool act) {
         constexpr int NR = decltype(nr_tag)::value;
-        const long long pv = P / VW;
-        V a[NR];
-#pragma unroll
-        for (int u = 0; u < NR; ++u) a[u] = ldv(at + u * pv);
 #pragma unroll
         for (int t0 = 0; t0 < K; t0 += VW) {
             if (t0 >= kk) break;
@@ -551,7 +564,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         // tasks of 32 vectors x RB rows, taken by the warps in turn; the pivot
         // rows' entries in registers
         const int nchunk = (nact + 31) / 32;
-        int S = nchunk > 0 ? (6 * nw + nchunk - 1) / nchunk : 1;
+        int S = nchunk > 0 ? ((sizeof(T) == 8 ? 6 : 12) * nw + nchunk - 1) / nchunk : 1;
         S = max(1, min(S, (R + RS - 1) / RS));
         const int RB = ((R + S - 1) / S + 1) / 2 * 2;
         S = RB > 0 ? (R + RB - 1) / RB : 0;
@@ -571,16 +584,44 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             int r = sub * RB;
             const int rb1 = min(R, r + RB);
             V *at = reinterpret_cast<V *>(Tab + (long long)(i0 + r) * P) + v;
-            const long long pv = P / VW;
-            if (RS == 8)
-                for (; r + 8 <= rb1; r += 8, at += 8 * pv)
-                    panel_rows(std::integral_constant<int, 8>(), at, r, kk, pr, act);
-            for (; r + 4 <= rb1; r += 4, at += 4 * pv)
-                panel_rows(std::integral_constant<int, 4>(), at, r, kk, pr, act);
-            for (; r + 2 <= rb1; r += 2, at += 2 * pv)
-                panel_rows(std::integral_constant<int, 2>(), at, r, kk, pr, act);
-            for (; r < rb1; ++r, at += pv)
-                panel_rows(std::integral_constant<int, 1>(), at, r, kk, pr, act);
+            // RS rows at a time (with registers to spare the next RS in flight);
+            // then 4, 2 and 1
+            auto load_rows = [&](auto nr_tag, V(&x)[decltype(nr_tag)::value], const V *from) {
+#pragma unroll
+                for (int u = 0; u < decltype(nr_tag)::value; ++u) x[u] = ldv(from + u * pv);
+            };
+            const std::integral_constant<int, RS> rs;
+            V a[RS];
+            if constexpr (K == kPanelK) {
+                V b[RS];
+                if (r + RS <= rb1) load_rows(rs, a, at);
+                for (; r + RS <= rb1; r += RS, at += RS * pv) {
+                    const bool more = r + 2 * RS <= rb1;
+                    if (more) load_rows(rs, b, at + RS * pv);
+                    panel_rows(rs, a, at, r, kk, pr, act);
+                    if (more) {
+#pragma unroll
+                        for (int u = 0; u < RS; ++u) a[u] = b[u];
+                    }
+                }
+            } else {
+                for (; r + RS <= rb1; r += RS, at += RS * pv) {
+                    load_rows(rs, a, at);
+                    panel_rows(rs, a, at, r, kk, pr, act);
+                }
+            }
+            auto rest = [&](auto nr_tag) {
+                constexpr int NR = decltype(nr_tag)::value;
+                V c[NR];
+                if (r + NR > rb1) return;
+                load_rows(nr_tag, c, at);
+                panel_rows(nr_tag, c, at, r, kk, pr, act);
+                r += NR;
+                at += NR * pv;
+            };
+            if (RS == 8) rest(std::integral_constant<int, 4>());
+            rest(std::integral_constant<int, 2>());
+            rest(std::integral_constant<int, 1>());
         }
         // the other columns of marked rows
         if (!all && s_nflag) {
@@ -717,8 +758,12 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         Pick r;
         r.aux = r.zero = 0;
         // (the abort word is asked for a pivot ahead: it is in host memory)
-        const int ab = ab_next;
-        if (tid == 32 * kPollFirst) ab_next = abort_peek(abort_word);
+        int ab = ab_next;
+        if (tid == 32 * kPollFirst) {
+            ab_next = abort_peek(abort_word);
+            // (the wall-clock limit, in case the host is late with the word)
+            if (limit_ns > 0 && global_ns() - t_start > (unsigned long long)limit_ns) ab = 1;
+        }
         if (ab) {
             atomicExch(err, 1);
             s_fail[0] = 1;
@@ -1351,9 +1396,10 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
 template <typename T, bool DUAL>
 __global__ void __launch_bounds__(kPanelThreads, 1)
     panel_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
-                 unsigned nonce) {
+                 unsigned nonce, long long limit_ns) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    panel_solve<T, DUAL, kPanelK>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce, smem_raw);
+    panel_solve<T, DUAL, kPanelK>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce,
+                                  limit_ns, smem_raw);
 }
 
 // Many LPs in one launch.  items[] lists (lp, rank) pairs, the ranks of one LP
@@ -1380,10 +1426,10 @@ __global__ void __launch_bounds__(kPanelThreads, 2)
         LpDesc *d = descs + w.x;
         if (d->sense)
             panel_solve<T, true, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
-                                               smem_raw);
+                                               0, smem_raw);
         else
             panel_solve<T, false, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
-                                                smem_raw);
+                                                0, smem_raw);
     }
 }
 
@@ -1430,7 +1476,8 @@ cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long lo
                          long long budget, cudaStream_t s) {
     int drop = sh.drop;
     unsigned nonce = next_nonce();
-    void *args[] = {&d_desc, &spin_limit, &budget, &drop, &nonce};
+    long long limit_ns = sh.limit_ns;
+    void *args[] = {&d_desc, &spin_limit, &budget, &drop, &nonce, &limit_ns};
     const void *fn = prec == PREC_FP64 ? (sh.dual ? (const void *)panel_kernel<double, true>
                                                   : (const void *)panel_kernel<double, false>)
                                        : (sh.dual ? (const void *)panel_kernel<float, true>
