@@ -45,6 +45,18 @@ constexpr int kDistRows = 4;
 // vectors in place (lp_options.zero_skip)
 constexpr long long kSkipElems = 1ll << 25;
 
+// The panel kernel overlaps its panels with the selection (on a second tableau
+// buffer) from this many tableau elements on, and below this many per CTA.
+// Measured, us per pivot, in turn / overlapped: 512^2 (0.54 M elements) 7.3 /
+// 7.4, 700 x 900 (1.1 M) 7.6 / 7.5, 1024^2 8.3 / 7.8, 512 x 4096 10.9 / 8.6,
+// 4096 x 512 10.3 / 9.7, 1024 x 4096 14.3 / 10.8, 2048^2 13.7 / 10.3 (dual form
+// 16.1 / 12.3), 4096^2 (222 K elements per CTA) 35.7 / 33.2; on 50 CTAs 1024^2
+// 11.8 / 9.6, 2048^2 (169 K) 28.0 / 25.6, 3500^2 (491 K) 67.5 / 69.1; 8192^2
+// (885 K) 118 / 119, where the panels of 8 instead of 16 pivots cost more than
+// the selection they hide.
+constexpr long long kOverlapElems = 1ll << 20;
+constexpr long long kOverlapPerCta = 450000;
+
 struct lp_handle {
     lp_options opt;
     int device = 0;
@@ -388,29 +400,47 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     if (pmode == 1) pmode = (long long)M * P >= kBlockElems ? 4 : 2;
     // The automatic mode takes the panel kernel for every rule the LP needs,
     // where its shared memory and its workspace fit (a workspace above 64 MB
-    // only when the tableau is at least twice as large); then no second
-    // buffer is needed.  Not on wide LPs above 2^20 elements: every vector is
-    // updated there, and a CTA's few rows split unevenly (512 x 4096: 11.0 us
-    // per pivot against 10.8).
+    // only when the tableau is at least twice as large), with overlapped
+    // panels where they pay and the second buffer can be had.  Wide LPs from
+    // 2^20 elements, where no column is left out and a CTA's few rows split
+    // unevenly, only with overlapped panels (512 x 4096: 8.6 us per pivot; in
+    // turn 10.9, the two-pivot kernel 10.1).
     const int pdrop = h->opt.zero_skip == 2 || (h->opt.zero_skip == 1 && 4ll * m >= n);
-    const PivotShape psh = choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, (int)sense, pdrop);
+    auto panel_shape = [&](int rule, bool ov) {
+        return choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, rule, pdrop, ov);
+    };
+    const PivotShape psh = panel_shape((int)sense, false);
+    const long long elems = (long long)M * P;
     const size_t pws = panel_workspace(h->prec, m, N, P, psh.ctas, kPanelK);
-    bool panel = h->opt.pipeline == 1 &&
-                 (4ll * m >= n || (long long)M * P < (1ll << 20)) && (pws <= (64ull << 20) || 2 * pws <= tbytes) &&
-                 psh.pipe == 4;
+    bool panel = h->opt.pipeline == 1 && psh.pipe == 4 &&
+                 (pws <= (64ull << 20) || 2 * pws <= tbytes);
+    bool overlap = panel && h->prec == PREC_FP64 && elems >= kOverlapElems &&
+                   elems < kOverlapPerCta * psh.ctas && panel_shape((int)sense, true).pipe == 5;
+    panel = panel && (4ll * m >= n || elems < (1ll << 20) || overlap);
     if (panel && h->region) {
         // (what the buffers below take besides the inputs, with slack)
-        const size_t need = tbytes + pws + (size_t)(m + n) * 16 +
-                            64 * (size_t)h->sms * sizeof(Cand) + (64u << 10);
-        panel = h->region_size - h->region_used >= need;
+        size_t need = tbytes + pws + (size_t)(m + n) * 16 +
+                      64 * (size_t)h->sms * sizeof(Cand) + (64u << 10);
+        if (h->prec == PREC_FP32) {  // and the reinversions'
+            const size_t ns = (size_t)std::min(m, n), cap = (size_t)std::max(m, n) + m;
+            need += cap * (6 * sizeof(int) + 4 * sizeof(double)) +
+                    ns * ((2 * ns + 1 + 31) / 32 * 32) * sizeof(double);
+        }
+        const size_t room = h->region_size - h->region_used;
+        overlap = overlap && room >= need + tbytes + 256;
+        panel = room >= need;
     }
     if (panel && grow_bytes(h, &h->dpanel, &h->cap_panel, pws) != cudaSuccess) {
         cudaGetLastError();
         panel = false;
     }
+    if (overlap && (!panel || grow_bytes(h, &h->dT2, &h->cap_T2, tbytes) != cudaSuccess)) {
+        if (panel) cudaGetLastError();
+        overlap = false;
+    }
     if (panel) pmode = 0;
     const bool dwant = dualr && h->opt.pipeline != 0 && !panel;
-    bool have_t2 = false;
+    bool have_t2 = overlap;
     if (pmode >= 3 || dwant) {
         have_t2 = grow_bytes(h, &h->dT2, &h->cap_T2, (size_t)M * P * esz) == cudaSuccess;
         if (!have_t2) cudaGetLastError();
@@ -439,7 +469,7 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     const int split = skip ? n / sector * sector : 0;
     auto shape_for = [&](int rule) {
         if (panel)
-            return choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, rule, pdrop);
+            return panel_shape(rule, overlap);
         if (rule == 0 && pmode) {
             PivotShape ps = choose_pipe_shape(h->prec, M, P, h->sms, h->opt.threads, h->opt.ctas,
                                               pmode == 4 ? 2 : 0, pmode == 4 ? split : 0);
@@ -604,7 +634,7 @@ namespace {
 // The words a pivot launch wants zeroed: the synchronisation block, and the
 // records of the panel kernel.
 size_t bar_bytes(const PivotShape &sh) {
-    return (kBarWords + (sh.pipe == 4 ? kPanelRecWords : 0)) * sizeof(unsigned);
+    return (kBarWords + (sh.pipe >= 4 ? kPanelRecWords : 0)) * sizeof(unsigned);
 }
 
 // Start the wall-clock limit of a solve: lower the abort word (no kernel of

@@ -91,7 +91,7 @@ struct PivotShape {
     int use_smem = 0;              // selection scratch in shared memory (else global)
     int dual = 0;                  // dual simplex kernel (else primal)
     int pipe = 0;                  // pipelined kernel: 1 in place, 2 double-buffered, 3 two pivots per pass,
-                                   // 4 the panel kernel
+                                   // 4 the panel kernel, 5 with overlapped panels
     int sel_warps = 4;             // two pivots per pass: selection warps per CTA (4 or 8)
     int dist = 0;                  // two pivots per pass, primal: ratio test distributed over the CTAs
     int split = 0;                 // two pivots per pass, primal: first column of every CTA's second
@@ -115,6 +115,8 @@ constexpr int kBarWords = 256;
 // at most.  Its two record exchanges (a 128-byte line per CTA and exchange) follow
 // the synchronisation block and are zeroed with it before each launch.
 constexpr int kPanelK = 16, kPanelBatchK = 8;
+constexpr int kPanelOverlapK = 8;  // and as many of the panel being applied
+static_assert(2 * kPanelOverlapK == kPanelK, "the overlapped panels use the same slots");
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxCtas = 192;
 constexpr int kPanelRecWords = 2 * kPanelMaxCtas * 32;
@@ -168,9 +170,10 @@ cudaError_t launch_pivot_pipe(int prec, LpDesc *d_desc, const PivotShape &sh,
                               long long spin_limit, long long budget, cudaStream_t s);
 // The panel kernel's shape (pipe == 0: its shared memory does not fit), its
 // workspace bytes and its launch (gbs_panel.cu).
-PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop);
+PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop,
+                              bool overlap);
 size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K);
-size_t panel_smem(int prec, int m, int N, int G, int K);
+size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap = false);
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s);
 // The same over a batch's work items, panels of kPanelBatchK.

@@ -18,14 +18,20 @@
 // sub-partition, dependent or not (1.26 TFLOP/s in all), so a panel is bound
 // by its fmas once it carries about four pivots, the tableau moving once per
 // panel; the selection is a chain of two record exchanges and two dependent
-// round trips to L2 per pivot, about 6 us of latency.  The two alternate:
-// nothing streams while the chain runs, so its loads and its few FP64
-// instructions never queue behind the update's.  Measured, FP64, us per pivot,
-// against the kernels that update everything every one or two pivots: 256^2
-// 7.0 (was 9.3), 501 x 703 of the paper's family 6.7 (10.2), 512 x 4096 11.0
-// (10.8), 4096 x 512 10.4 (42), 2048^2 14.0 (22.4), its dual form 16.2 (22.9),
-// 8192^2 119 (136: 107 is its fmas at the FP64 peak); FP32 8192^2 21 (70).
-// Panels of 8 pivots instead of 16 were 1 to 4% slower from 512 x 4096 up.
+// round trips to L2 per pivot, about 6 us of latency.  On small tableaus, on
+// the largest and in FP32 the two alternate: nothing streams while the chain
+// runs, so its loads and its few FP64 instructions never queue behind the
+// panel's.  In between, where neither is small beside the other, panels of 8
+// run on eight more warps and a second buffer while the next one's pivots are
+// selected (OV below): the chain takes about 9 us then, the panel's time is
+// hidden.  Measured, FP64, us per pivot, against the kernels that update
+// everything every one or two pivots: 256^2 6.9 (was 9.3), 501 x 703 of the
+// paper's family 6.6 (10.2), 512 x 4096 8.6 (10.8; in turn 10.9), 4096 x 512
+// 9.7 (42; 10.3), 2048^2 10.3 (22.4; 13.7), its dual form 12.3 (22.9; 16.1),
+// 4096^2 33 (59; 36), 8192^2 118 (136; overlapped 119; 107 is its fmas at the
+// FP64 peak); FP32 8192^2 16 (70).  In turn, panels of 8 pivots instead of 16
+// were 1 to 4% slower from 512 x 4096 up; overlapped, four or six warps for the
+// panels were slower than eight from 2048^2 up (13.2 and 10.4 us).
 //
 // Work split (G CTAs).  CTA g owns
 //   the columns J_g (a contiguous strip) of the objective row and of every
@@ -293,12 +299,14 @@ __device__ __forceinline__ T fma_chain(T v, int k, const T *c, const T *p) {
 // Shared-memory layout of a CTA, shared by the kernel and the host's sizing.
 struct PanelLayout {
     int R, W, nvec, nwords;
-    size_t zs, prs, cs, rh, bas, lastp, rowz, bb, stay, list, total;
+    size_t zs, prs, cs, rh, bas, lastp, rowz, bb, stay, prev, out, list, total;
 };
 
-__host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz, int vw, int K) {
+// (slots: pending pivots at most; ov: with the bitmaps of the overlapped panels)
+__host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz, int vw, int slots,
+                                                    bool ov) {
     PanelLayout L;
-    const int stride = entry_stride(esz, K);
+    const int stride = entry_stride(esz, slots);
     L.R = (m + G - 1) / G + 1;  // slices differ by at most one row
     L.W = (N + G - 1) / G + 1;
     L.nvec = (N + vw - 1) / vw;
@@ -318,6 +326,8 @@ __host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz
     L.rowz = take((size_t)L.R);
     L.bb = take((size_t)L.nwords * sizeof(unsigned));
     L.stay = take((size_t)L.nwords * sizeof(unsigned));
+    L.prev = take(ov ? (size_t)L.nwords * sizeof(unsigned) : 0);
+    L.out = take(ov ? (size_t)L.nwords * sizeof(unsigned) : 0);
     L.list = take((size_t)L.nvec * sizeof(int));
     L.total = at;
     return L;
@@ -342,9 +352,21 @@ constexpr unsigned kFlagAll = 1u << 31;   // this panel gets every column
 constexpr unsigned kFlagZero = 1u << 30;  // the ratio rounds to zero
 constexpr unsigned kFlagWide = 1u << 29;  // a ratio key out of range
 
+// Overlapped panels: what the other warps do next.
+enum : int { kJobEnd = 0, kJobCopy = 1, kJobPanel = 2, kJobInPlace = 3 };
+
 // One LP on a group of G co-resident CTAs, this one its g-th, with panels of up
 // to K pivots.
-template <typename T, bool DUAL, int K>
+//
+// OV: panels overlapped with the selection.  The CTA has eight more warps,
+// which apply one panel from the current tableau buffer into the other while
+// the first eight select the next panel's pivots on the current one, with the
+// pivots of both panels pending.  The buffers change places when every CTA's
+// panel is done, which its next record 1 says.  A column that did not change
+// in this panel and the one before is the same in both buffers and is left
+// out; the launch starts by copying the tableau (under the first panel's
+// selection) and ends by applying the last pivots in place.
+template <typename T, bool DUAL, int K, bool OV>
 __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g,
                                             long long spin_limit, long long budget, int drop,
                                             unsigned nonce, long long limit_ns,
@@ -352,34 +374,37 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     typedef typename Vec<T>::type V;
     typedef typename DivisorOf<T>::type Divisor;
     constexpr int VW = Vec<T>::W;
-    constexpr int B = kPanelThreads, nw = kWarps, KS = entry_stride(sizeof(T), K);
-    constexpr int RS = sizeof(T) == 8 || K < kPanelK ? 4 : 8;  // rows of a panel step per warp
+    constexpr int NS = OV ? 2 * K : K;  // slots of pending pivots
+    constexpr int B = kPanelThreads, nw = kWarps, KS = entry_stride(sizeof(T), NS);
+    constexpr int RS = sizeof(T) == 8 || NS < kPanelK ? 4 : 8;  // rows of a panel step per warp
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ Slot s_loc[nw], s_ex1[kPollWarps], s_ex2[kPollWarps], s_ex3[kPollWarps];
     __shared__ __align__(16) T s_at[nw][KS];  // a warp's pending entries at one row or column
     __shared__ int s_flag, s_fail[2], s_nflag, s_task, s_scan[nw];
-    __shared__ int s_prow[K];  // pivot rows of the pending pivots
+    __shared__ int s_prow[NS];  // pivot rows of the pending pivots
+    __shared__ int s_job[5], s_done;  // OV: the panel to apply, panels applied
     __shared__ ulonglong2 s_rec[2];
     __shared__ unsigned long long s_aux[2][2][4];
 
     const int tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
-    T *const Tab = reinterpret_cast<T *>(d->T);
+    T *const bufs[2] = {reinterpret_cast<T *>(d->T), reinterpret_cast<T *>(OV ? d->T2 : d->T)};
+    T *Tab = bufs[0];  // the tableau of the last panel applied
     const long long P = d->P;
     const int m = d->m, N = d->N;
     const long long Mp = tag_pitch(m), Np = tag_pitch(N);
-    // pending columns (K x Mp) and rows (K x Np) and the records' further values
+    // pending columns (NS x Mp) and rows (NS x Np) and the records' further values
     // (by pivot parity, 2 exchanges x G x 4) as 16-byte values with the tag of their pivot, for
     // single entries (with one CTA they are all in its shared memory); and the
     // rows plain, for the panels
     ulonglong2 *const CT = reinterpret_cast<ulonglong2 *>(d->panel);
-    ulonglong2 *const PT = CT + (G > 1 ? K * Mp : 0);
-    ulonglong2 *const AX = PT + (G > 1 ? K * Np : 0);
+    ulonglong2 *const PT = CT + (G > 1 ? NS * Mp : 0);
+    ulonglong2 *const AX = PT + (G > 1 ? NS * Np : 0);
     T *const PR = reinterpret_cast<T *>(AX + (G > 1 ? 16 * G : 0));
     ulonglong2 *const recs = reinterpret_cast<ulonglong2 *>(d->recs);
     int *const err = d->err;
 
-    const PanelLayout L = panel_layout(m, N, G, sizeof(T), VW, K);
+    const PanelLayout L = panel_layout(m, N, G, sizeof(T), VW, NS, OV);
     T *const zs = reinterpret_cast<T *>(smem_raw + L.zs);
     T *const prs = reinterpret_cast<T *>(smem_raw + L.prs);
     T *const cs = reinterpret_cast<T *>(smem_raw + L.cs);
@@ -389,7 +414,14 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     unsigned char *const rowz = smem_raw + L.rowz;
     unsigned *const bb = reinterpret_cast<unsigned *>(smem_raw + L.bb);      // basic columns
     unsigned *const stay = reinterpret_cast<unsigned *>(smem_raw + L.stay);  // basic since the last panel
+    unsigned *const prev = reinterpret_cast<unsigned *>(smem_raw + L.prev);  // OV: in the panel before
+    unsigned *const out = reinterpret_cast<unsigned *>(smem_raw + L.out);    // OV: left out of the panel
     int *const list = reinterpret_cast<int *>(smem_raw + L.list);
+    // every selection thread (OV: half of the CTA)
+    auto cta_sync = [&]() {
+        if (OV) group_sync(5, nw);
+        else __syncthreads();
+    };
     const int nvec = L.nvec, nwords = L.nwords;
 
     const int i0 = (int)((long long)m * g / G), R = (int)((long long)m * (g + 1) / G) - i0;
@@ -418,7 +450,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     const long long trace_cap = d->trace_cap;
 
     // ------------------------------------------------------------- start --
-    {
+    if (!OV || tid < B) {
         const T *z = Tab + (long long)m * P;
         for (int c = tid; c < W; c += B) zs[c] = lds(z + c0 + c);
         for (int r = tid; r < R; r += B) {
@@ -430,28 +462,30 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         for (int w = tid; w < nwords; w += B) bb[w] = 0;
         // the padding of the last vector of the pending rows (other CTAs read
         // it once this CTA's records are out)
-        if (g == 0 && tid < K)
+        if (g == 0 && tid < NS)
             for (int j = N; j < nvec * VW; ++j) __stcg(PR + tid * P + j, (T)0);
         __threadfence();
         if (tid == 0) {
             s_fail[0] = s_fail[1] = 0;
             s_nflag = 0;
+            s_done = 0;
         }
-        __syncthreads();
+        cta_sync();
         for (int i = tid; i < m; i += B) {
             const int j = __ldcg(d->basis + i);
             atomicOr(&bb[j >> 5], 1u << (j & 31));
         }
-        __syncthreads();
+        cta_sync();
         for (int w = tid; w < nwords; w += B) {
             // (columns past the last one never need an update)
             if (w == nwords - 1 && (N & 31)) bb[w] |= ~0u << (N & 31);
             stay[w] = bb[w];
+            if (OV) prev[w] = ~0u;  // (the copy makes the buffers equal)
         }
         if (scan) {
             // rows whose entries in basic columns are not all +0 (but the
             // unit entry): -0 from the dual rule or a refresh
-            __syncthreads();
+            cta_sync();
             for (int r = wid; r < R; r += nw) {
                 const T *row = Tab + (long long)(i0 + r) * P;
                 int bad = 0;
@@ -472,10 +506,15 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 }
             }
         }
-        __syncthreads();
+        cta_sync();
     }
 
-    int k = 0;            // pending pivots
+    int k = 0;            // pending pivots of this panel
+    int kold = 0;         // OV: and of the panel that is being applied,
+    int ho = 0, hn = 0;   // in the slots from ho; this panel's from hn
+    int cur = 0, jobs = 0;
+    // the slot of the pos-th pending pivot, oldest first
+    auto slot = [&](int pos) { return !OV ? pos : pos < kold ? ho + pos : hn + pos - kold; };
     unsigned epoch = 1;   // number of the pivot whose records are awaited
     unsigned ecur = 1;    // number of the pivot being made
     int nodrop = 0;       // this panel gets every column
@@ -485,7 +524,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
 
     // NR rows of one 16-byte vector column: kk pending pivots on each.
     const long long pv = P / VW;
-    auto panel_rows = [&](auto nr_tag, V(&a)[decltype(nr_tag)::value], V *at, int r, int kk,
+    auto panel_rows = [&](auto nr_tag, V(&a)[decltype(nr_tag)::value], V *at, int r, int h, int kk,
                           const V(&pr)[K], bool act) {
         constexpr int NR = decltype(nr_tag)::value;
 #pragma unroll
@@ -494,11 +533,11 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             V c[NR];
 #pragma unroll
             for (int u = 0; u < NR; ++u)
-                c[u] = *reinterpret_cast<const V *>(cs + (r + u) * KS + t0);
+                c[u] = *reinterpret_cast<const V *>(cs + (r + u) * KS + h + t0);
 #pragma unroll
             for (int t = t0; t < t0 + VW; ++t) {
                 if (t >= kk) break;
-                const int lp = s_prow[t] - i0 - r;
+                const int lp = s_prow[h + t] - i0 - r;
                 if ((unsigned)lp < (unsigned)NR) {
 #pragma unroll
                     for (int u = 0; u < NR; ++u) {
@@ -518,23 +557,26 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         }
     };
 
-    // Apply the kk pending pivots to this CTA's rows.
-    auto apply_panel = [&](int kk) {
+    // Apply the kk pending pivots in the slots from h to this CTA's rows, from
+    // src to dst, but to the columns in the bitmap `left_out` (none with `all`)
+    // only on marked rows.  Thread bt of nw warps; sync() is their barrier.
+    auto panel_job = [&](const T *src, T *dst, int h, int kk, bool all, const unsigned *left_out,
+                         int bt, auto &&sync) {
+        const int bw = bt >> 5;
         // the vectors to update, in order
         int nact;
-        const bool all = !drop || nodrop;
         constexpr unsigned full = (1u << VW) - 1u;
-        if (tid == 0) s_task = 0;
+        if (bt == 0) s_task = 0;
         if (all) {
-            for (int v = tid; v < nvec; v += B) list[v] = v;
+            for (int v = bt; v < nvec; v += B) list[v] = v;
             nact = nvec;
-            __syncthreads();
+            sync();
         } else {
             const int per = (nwords + B - 1) / B;
-            const int w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
+            const int w0 = min(nwords, bt * per), w1 = min(nwords, w0 + per);
             int cnt = 0;
             for (int w = w0; w < w1; ++w) {
-                const unsigned s = stay[w];
+                const unsigned s = left_out[w];
                 for (int u = 0; u < 32 / VW; ++u) cnt += (s >> (u * VW) & full) != full;
             }
             int pre = cnt;
@@ -543,21 +585,21 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 const int y = __shfl_up_sync(kAll, pre, o);
                 if (lane >= o) pre += y;
             }
-            if (lane == 31) s_scan[wid] = pre;
-            __syncthreads();
+            if (lane == 31) s_scan[bw] = pre;
+            sync();
             int base = 0;
             nact = 0;
             for (int w = 0; w < nw; ++w) {
-                if (w < wid) base += s_scan[w];
+                if (w < bw) base += s_scan[w];
                 nact += s_scan[w];
             }
             int at = base + pre - cnt;
             for (int w = w0; w < w1; ++w) {
-                const unsigned s = stay[w];
+                const unsigned s = left_out[w];
                 for (int u = 0; u < 32 / VW; ++u)
                     if ((s >> (u * VW) & full) != full) list[at++] = w * (32 / VW) + u;
             }
-            __syncthreads();
+            sync();
         }
         upd += (unsigned long long)(all ? P / VW : nact) * kk;
         left += (unsigned long long)(all ? 0 : P / VW - nact) * kk;
@@ -580,44 +622,46 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             V pr[K];
 #pragma unroll
             for (int t = 0; t < K; ++t)
-                if (t < kk) pr[t] = ldv(reinterpret_cast<const V *>(PR + t * P) + v);
+                if (t < kk) pr[t] = ldv(reinterpret_cast<const V *>(PR + (h + t) * P) + v);
             int r = sub * RB;
             const int rb1 = min(R, r + RB);
-            V *at = reinterpret_cast<V *>(Tab + (long long)(i0 + r) * P) + v;
+            const V *from = reinterpret_cast<const V *>(src + (long long)(i0 + r) * P) + v;
+            V *at = reinterpret_cast<V *>(dst + (long long)(i0 + r) * P) + v;
             // RS rows at a time (with registers to spare the next RS in flight);
             // then 4, 2 and 1
-            auto load_rows = [&](auto nr_tag, V(&x)[decltype(nr_tag)::value], const V *from) {
+            auto load_rows = [&](auto nr_tag, V(&x)[decltype(nr_tag)::value], const V *q) {
 #pragma unroll
-                for (int u = 0; u < decltype(nr_tag)::value; ++u) x[u] = ldv(from + u * pv);
+                for (int u = 0; u < decltype(nr_tag)::value; ++u) x[u] = ldv(q + u * pv);
             };
             const std::integral_constant<int, RS> rs;
             V a[RS];
-            if constexpr (K == kPanelK) {
+            if constexpr (NS == kPanelK) {
                 V b[RS];
-                if (r + RS <= rb1) load_rows(rs, a, at);
-                for (; r + RS <= rb1; r += RS, at += RS * pv) {
+                if (r + RS <= rb1) load_rows(rs, a, from);
+                for (; r + RS <= rb1; r += RS, at += RS * pv, from += RS * pv) {
                     const bool more = r + 2 * RS <= rb1;
-                    if (more) load_rows(rs, b, at + RS * pv);
-                    panel_rows(rs, a, at, r, kk, pr, act);
+                    if (more) load_rows(rs, b, from + RS * pv);
+                    panel_rows(rs, a, at, r, h, kk, pr, act);
                     if (more) {
 #pragma unroll
                         for (int u = 0; u < RS; ++u) a[u] = b[u];
                     }
                 }
             } else {
-                for (; r + RS <= rb1; r += RS, at += RS * pv) {
-                    load_rows(rs, a, at);
-                    panel_rows(rs, a, at, r, kk, pr, act);
+                for (; r + RS <= rb1; r += RS, at += RS * pv, from += RS * pv) {
+                    load_rows(rs, a, from);
+                    panel_rows(rs, a, at, r, h, kk, pr, act);
                 }
             }
             auto rest = [&](auto nr_tag) {
                 constexpr int NR = decltype(nr_tag)::value;
                 V c[NR];
                 if (r + NR > rb1) return;
-                load_rows(nr_tag, c, at);
-                panel_rows(nr_tag, c, at, r, kk, pr, act);
+                load_rows(nr_tag, c, from);
+                panel_rows(nr_tag, c, at, r, h, kk, pr, act);
                 r += NR;
                 at += NR * pv;
+                from += NR * pv;
             };
             if (RS == 8) rest(std::integral_constant<int, 4>());
             rest(std::integral_constant<int, 2>());
@@ -627,26 +671,106 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         if (!all && s_nflag) {
             for (int r = 0; r < R; ++r) {
                 if (!rowz[r]) continue;
-                V *const row = reinterpret_cast<V *>(Tab + (long long)(i0 + r) * P);
-                for (int v = tid; v < nvec; v += B) {
+                const V *const from = reinterpret_cast<const V *>(src + (long long)(i0 + r) * P);
+                V *const to = reinterpret_cast<V *>(dst + (long long)(i0 + r) * P);
+                for (int v = bt; v < nvec; v += B) {
                     const int j = v * VW;
-                    if ((stay[j >> 5] >> (j & 31) & full) != full) continue;
-                    V x = ldv(row + v);
+                    if ((left_out[j >> 5] >> (j & 31) & full) != full) continue;
+                    V x = ldv(from + v);
                     for (int t = 0; t < kk; ++t) {
-                        const V pt = ldv(reinterpret_cast<const V *>(PR + t * P) + v);
-                        if (s_prow[t] == i0 + r) x = pt;
-                        else vfma(x, cs[r * KS + t], pt);
+                        const V pt = ldv(reinterpret_cast<const V *>(PR + (h + t) * P) + v);
+                        if (s_prow[h + t] == i0 + r) x = pt;
+                        else vfma(x, cs[r * KS + h + t], pt);
                     }
-                    row[v] = x;
+                    to[v] = x;
                 }
             }
         }
-        __syncthreads();  // stay was read
+        __threadfence();  // other CTAs read these rows after this CTA's next record
+        sync();
+    };
+    // The pending pivots of a full or last panel, in place (not OV).
+    auto apply_panel = [&](int kk) {
+        panel_job(Tab, Tab, 0, kk, !drop || nodrop, stay, tid, cta_sync);
         for (int w = tid; w < nwords; w += B) stay[w] = bb[w];
         for (int r = tid; r < R; r += B) lastp[r] = -1;
         nodrop = 0;
-        __threadfence();  // other CTAs read these rows after this CTA's next record
-        __syncthreads();
+        cta_sync();
+    };
+
+    // OV, the other eight warps: jobs as the selection warps post them.
+    if (OV && tid >= B) {
+        const int bt = tid - B;
+        auto sync = [&]() { group_sync(6, nw); };
+        for (int done = 1;; ++done) {
+            group_sync(7, 2 * nw);
+            const int kind = s_job[0];
+            if (kind == kJobEnd) break;
+            if (kind == kJobCopy) {
+                const V *src = reinterpret_cast<const V *>(bufs[0] + (long long)i0 * P);
+                V *dst = reinterpret_cast<V *>(bufs[1] + (long long)i0 * P);
+                const long long cnt = (long long)R * pv;
+#pragma unroll 4
+                for (long long e = bt; e < cnt; e += B) dst[e] = ldv(src + e);
+                __threadfence();
+                sync();
+            } else {
+                T *const src = bufs[s_job[3]];
+                panel_job(src, kind == kJobPanel ? bufs[s_job[3] ^ 1] : src, s_job[1], s_job[2],
+                          s_job[4] != 0, out, bt, sync);
+            }
+            if (bt == 0) *(volatile int *)&s_done = done;
+        }
+        if (g == 0 && bt == 0 && d->work) {
+            d->work[0] += upd;
+            d->work[1] += left;
+        }
+        return;
+    }
+    // OV: post a job (every selection thread).
+    auto post = [&](int kind, int h, int kk, bool all) {
+        if (tid == 0) {
+            s_job[0] = kind, s_job[1] = h, s_job[2] = kk, s_job[3] = cur, s_job[4] = all;
+        }
+        cta_sync();
+        group_arrive(7, 2 * nw);
+        ++jobs;
+    };
+    // OV: wait for the jobs posted; they have no waits of their own.
+    auto wait_jobs = [&]() {
+        if (lane == 0)
+            while (*(volatile int *)&s_done != jobs) {
+            }
+        __syncwarp();
+    };
+    // Every CTA of the group; false when a wait ran out.
+    auto group_barrier = [&]() {
+        if (!OV) return grid_sync(d->bar, err, G, spin_limit, &s_flag);
+        cta_sync();
+        if (tid == 0) {
+            int ok = 1;
+            if (G > 1) {
+                const unsigned g0 = ld_acquire(d->bar + 32);
+                __threadfence();
+                if (atom_add_acq_rel(d->bar, 1u) == (unsigned)G - 1u) {
+                    atomicExch(d->bar, 0u);
+                    st_release(d->bar + 32, g0 + 1u);
+                } else {
+                    const long long t0 = clock64();
+                    while (ld_acquire(d->bar + 32) == g0) {
+                        if (clock64() - t0 > spin_limit || *(volatile int *)err) {
+                            atomicExch(err, 1);
+                            break;
+                        }
+                    }
+                }
+                __threadfence();
+            }
+            if (*(volatile int *)err) ok = 0;
+            s_flag = ok;
+        }
+        cta_sync();
+        return s_flag != 0;
     };
 
     // A value written by another CTA, once it carries the tag of pivot e.
@@ -685,7 +809,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         else st_half(recs + (which * G + g) * kRec, x, ix, epoch);
     };
     // One round trip for what a warp needs of this pivot: pending entries
-    // (lane t < k: pend + t * step, or own[t] where there is one CTA) into its
+    // (lane t: slot t's at pend + t * step, or own[t] with one CTA) into its
     // s_at, and in the lanes below the further values of cta1's record 1 and
     // cta2's record 2 (-1: not wanted).  A value is waited for until it
     // carries its pivot's tag: it was stored before a record already seen, so
@@ -694,9 +818,10 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     auto fetch = [&](const ulonglong2 *pend, long long step, const T *own, int cta1, int cta2,
                      int fail) {
         unsigned long long v = 0;
-        const bool pnd = own != nullptr && lane < k;
+        const int npend = kold + k, sl = slot(lane);
+        const bool pnd = own != nullptr && lane < npend;
         if (G == 1) {
-            v = pnd ? to_bits(own[lane]) : s_aux[ecur & 1][lane >= kNum2][lane & 3];
+            v = pnd ? to_bits(own[sl]) : s_aux[ecur & 1][lane >= kNum2][lane & 3];
         } else {
             // (one address per lane, kept apart from how it was chosen: three
             // branches with a load each would wait for three round trips)
@@ -706,11 +831,11 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 at = (unsigned long long)(further_at(e, 0, cta1) + lane - kRhs1);
             if (cta2 >= 0 && lane >= kNum2 && lane <= kRcp2)
                 at = (unsigned long long)(further_at(e, 1, cta2) + lane - kNum2);
-            if (pnd) at = (unsigned long long)(pend + lane * step), e = ecur - k + lane;
+            if (pnd) at = (unsigned long long)(pend + sl * step), e = ecur - npend + lane;
             asm volatile("" : "+l"(at), "+r"(e));
             if (at) v = tagged(reinterpret_cast<const ulonglong2 *>(at), e, fail);
         }
-        if (pnd) s_at[wid][lane] = from_bits<T>(v);
+        if (pnd) s_at[wid][sl] = from_bits<T>(v);
         __syncwarp();
         return v;
     };
@@ -769,7 +894,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             s_fail[0] = 1;
         }
         if (G == 1) {
-            __syncthreads();
+            cta_sync();
             const unsigned ix = (unsigned)s_rec[0].y;
             r.x = s_rec[0].x;
             r.idx = (int)(ix & kIdxMask) - 1;
@@ -802,7 +927,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 s.vk = vk, s.key = key, s.idx = idx, s.x = x, s.src = e, s.flag = flag;
             }
         }
-        __syncthreads();
+        cta_sync();
         int w = 0;
         unsigned long long bv = s_ex1[0].vk;
         int bk = s_ex1[0].key, fl = s_ex1[0].flag;
@@ -827,7 +952,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         Pick r;
         r.x = 0;
         if (G == 1) {
-            __syncthreads();
+            cta_sync();
             const unsigned ix = (unsigned)s_rec[1].y;
             r.aux = (int)(s_rec[1].x >> 32);
             r.idx = (int)(ix & kIdxMask) - 1;
@@ -868,7 +993,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 s.src = e0 + at * 32 * kPollWarps;
             }
         }
-        __syncthreads();
+        cta_sync();
         r.idx = -1;
         r.aux = r.zero = r.cta = 0;
         int w = 0;
@@ -914,7 +1039,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                     s.vk = ek, s.key = key, s.idx = (int)ix, s.aux = aux, s.src = e;
                 }
             }
-            __syncthreads();
+            cta_sync();
             win = s_ex3;
 #pragma unroll
             for (int q = 1; q < kPollWarps; ++q)
@@ -1023,7 +1148,12 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         return at;
     };
 
-    // Column q on this CTA's rows (row warps), the k pending pivots applied to
+    // The pending pivots on one entry.
+    auto pending_chain = [&](T v, const T *c, const T *q) {
+        if (OV && kold > 0) v = fma_chain(v, kold, c + ho, q + ho);
+        return fma_chain(v, k, c + hn, q + hn);
+    };
+    // Column q on this CTA's rows (row warps), the pending pivots applied to
     // the tableau of the last panel.  Returns whether an entry is not finite.
     // f: what fetch() returned, for the caller.
     auto form_col = [&](int q, int cta1, int cta2, int which, unsigned long long *f) {
@@ -1038,14 +1168,18 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             const int lp = lastp[rr];
             const T *c = cs + rr * KS;
             if (!__any_sync(kAll, lp >= 0)) {
-                v = fma_chain(v, k, c, s_at[wid]);
+                v = pending_chain(v, c, s_at[wid]);
             } else {  // a row that was a pivot row starts from that pivot's row
                 if (lp >= 0) v = s_at[wid][lp];
-                for (int t = lp + 1; t < k; ++t) v = pfma(-c[t], s_at[wid][t], v);
+                int pos = lp < 0 ? 0 : 1 + (OV && kold > 0 && (lp & K) == ho ? lp - ho : kold + lp - hn);
+                for (; pos < kold + k; ++pos) {
+                    const int t = slot(pos);
+                    v = pfma(-c[t], s_at[wid][t], v);
+                }
             }
             if (r < R) {
-                cs[r * KS + k] = v;
-                if (G > 1) st_half(CT + k * Mp + i0 + r, to_bits(v), ecur, nonce);
+                cs[r * KS + hn + k] = v;
+                if (G > 1) st_half(CT + (hn + k) * Mp + i0 + r, to_bits(v), ecur, nonce);
                 bad |= not_finite(v);
             }
         }
@@ -1053,20 +1187,25 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         return bad;
     };
     // An entry of row p (column c of the strip), from its value v in the last
-    // panel's tableau; tp: the last pending pivot with pivot row p, or -1.
+    // panel's tableau; tp: the position of the last pending pivot with pivot row
+    // p, or -1.
     auto form_row_elem = [&](T v, int tp, int c) {
         const T *pr = prs + c * KS;
-        if (tp < 0) return fma_chain(v, k, pr, s_at[wid]);
-        v = pr[tp];
-        for (int t = tp + 1; t < k; ++t) v = pfma(-s_at[wid][t], pr[t], v);
+        if (tp < 0) return pending_chain(v, s_at[wid], pr);
+        v = pr[slot(tp)];
+        for (int pos = tp + 1; pos < kold + k; ++pos) {
+            const int t = slot(pos);
+            v = pfma(-s_at[wid][t], pr[t], v);
+        }
         return v;
     };
     auto last_pending = [&](int p) {
-        const unsigned b = __ballot_sync(kAll, lane < k && s_prow[lane & (K - 1)] == p);
+        const unsigned b =
+            __ballot_sync(kAll, lane < kold + k && s_prow[slot(lane) & (NS - 1)] == p);
         return 31 - __clz((int)b);
     };
-    // The rhs and the basis on this CTA's rows (row warps): pivot number kk of
-    // the panel, row p, entering column q.
+    // The rhs and the basis on this CTA's rows (row warps): the pivot in slot kk,
+    // row p, entering column q.
     auto update_rhs = [&](int kk, int p, int q, T rhs_p, const Divisor &dv) {
         if (rt - lane >= R) return;
         const T rp = dv.div(rhs_p);
@@ -1114,6 +1253,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     };
 
     // ------------------------------------------------------------- pivots --
+    if (OV) post(kJobCopy, 0, 0, false);
     if (!DUAL && col_warp) {
         const bool bland = deg >= bland_after;
         unsigned long long vk = ~0ull;
@@ -1149,12 +1289,32 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             break;
         }
         if (k == K) {
-            apply_panel(k);
-            k = 0;
-            // (the dual rule reads other CTAs' rows next)
-            if (DUAL && !grid_sync(d->bar, err, G, spin_limit, &s_flag)) {
-                status = ST_TIMEOUT;
-                break;
+            if constexpr (OV) {
+                // every CTA's panel (or copy) is done: its record says so
+                if (jobs > 1) cur ^= 1, Tab = bufs[cur];
+                const bool all = !drop || nodrop;
+                for (int w = tid; w < nwords; w += B) {
+                    const unsigned s = stay[w];
+                    out[w] = prev[w] & s;
+                    prev[w] = all ? 0u : s;
+                    stay[w] = bb[w];
+                }
+                for (int r = tid; r < R; r += B)  // (the other half's slots are used again)
+                    if (lastp[r] >= 0 && (lastp[r] & K) != hn) lastp[r] = -1;
+                ho = hn;
+                hn ^= K;
+                kold = K;
+                k = 0;
+                nodrop = 0;
+                post(kJobPanel, ho, K, all);
+            } else {
+                apply_panel(k);
+                k = 0;
+                // (the dual rule reads other CTAs' rows next)
+                if (DUAL && !group_barrier()) {
+                    status = ST_TIMEOUT;
+                    break;
+                }
             }
         }
         int p, q, var = 0;            // leaving row, entering column, leaving variable
@@ -1170,7 +1330,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 bool wide = false;
                 int loc = -1;
                 for (int r = rt; r < R; r += B) {
-                    const T a = cs[r * KS + k];
+                    const T a = cs[r * KS + hn + k];
                     if (okey(a) <= lim_p) continue;
                     const unsigned sk = ratio_key(pos_part(rh[r]), a, &wide);
                     if (sk < sk1) sk2 = sk1, sk1 = sk, loc = r;
@@ -1180,25 +1340,25 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                     2, nw - 1 - wid, rw, sk1, sk2, loc, wide, bad,
                     [&](auto &&f) {
                         for (int r = rt; r < R; r += B) {
-                            const T a = cs[r * KS + k];
+                            const T a = cs[r * KS + hn + k];
                             bool w;
                             if (okey(a) > lim_p) f(r, ratio_key(pos_part(rh[r]), a, &w));
                         }
                     },
                     [&](int r, bool div, int *key) {
                         *key = bland ? bas[r] : i0 + r;
-                        return div ? okey(pos_part(rh[r]) / cs[r * KS + k]) : zero_k;
+                        return div ? okey(pos_part(rh[r]) / cs[r * KS + hn + k]) : zero_k;
                     },
                     [&](int r, unsigned sk, unsigned fl) {
                         publish(1, r < 0 ? 0ull : ((unsigned long long)(unsigned)bas[r] << 32) | sk,
                                 r < 0 ? -1 : i0 + r, fl);
                         if (r < 0) return;
                         set_further(1, 0, to_bits(rh[r]));
-                        set_further(1, 1, to_bits(cs[r * KS + k]));
+                        set_further(1, 1, to_bits(cs[r * KS + hn + k]));
                     });
                 open_gate(4);
                 // (the reciprocal follows while the records are exchanged)
-                if (mine >= 0) set_further(1, 2, to_bits(Divisor::recip(cs[mine * KS + k])));
+                if (mine >= 0) set_further(1, 2, to_bits(Divisor::recip(cs[mine * KS + hn + k])));
                 __syncwarp();
             }
         } else {
@@ -1221,7 +1381,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                     T v = q0 == ct - lane ? first : lds(Tab + (long long)p * P + j);
                     v = form_row_elem(v, tp, cc);
                     if (!act) continue;
-                    prs[c * KS + k] = v;
+                    prs[c * KS + hn + k] = v;
                     bad |= j != var && (stay[j >> 5] >> (j & 31) & 1u) && !is_zero(v);
                     if (j >= N - 1 || okey(v) >= lim_np) continue;
                     const unsigned sk = ratio_key(pos_part(zs[c]), neg(v), &wide);
@@ -1234,23 +1394,23 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                     [&](auto &&f) {
                         for (int c = ct; c < W; c += B) {
                             bool w;
-                            const T v = prs[c * KS + k];
+                            const T v = prs[c * KS + hn + k];
                             if (c0 + c < N - 1 && okey(v) < lim_np)
                                 f(c, ratio_key(pos_part(zs[c]), neg(v), &w));
                         }
                     },
                     [&](int c, bool div, int *key) {
                         *key = c0 + c;
-                        return div ? okey(pos_part(zs[c]) / neg(prs[c * KS + k])) : zero_k;
+                        return div ? okey(pos_part(zs[c]) / neg(prs[c * KS + hn + k])) : zero_k;
                     },
                     [&](int c, unsigned sk, unsigned fl) {
                         publish(1, sk, c < 0 ? -1 : c0 + c, fl);
                         if (c < 0) return;
                         set_further(1, 0, to_bits(zs[c]));
-                        set_further(1, 1, to_bits(prs[c * KS + k]));
+                        set_further(1, 1, to_bits(prs[c * KS + hn + k]));
                     });
                 open_gate(3);
-                if (mine >= 0) set_further(1, 2, to_bits(Divisor::recip(prs[mine * KS + k])));
+                if (mine >= 0) set_further(1, 2, to_bits(Divisor::recip(prs[mine * KS + hn + k])));
                 __syncwarp();
             }
         }
@@ -1316,14 +1476,14 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                     v = q0 == ct - lane ? first : lds(rowp + cc);
                     v = form_row_elem(v, tp, cc);
                 } else {
-                    v = prs[cc * KS + kc];
+                    v = prs[cc * KS + hn + kc];
                 }
                 if (!act) continue;
                 if (!DUAL) flag |= j != var && (stay[j >> 5] >> (j & 31) & 1u) && !is_zero(v);
                 const T pr = dv.div(v);
-                prs[c * KS + kc] = pr;
-                if (G > 1) st_half(PT + kc * Np + j, to_bits(pr), ecur, nonce);
-                __stcg(PR + kc * P + j, pr);
+                prs[c * KS + hn + kc] = pr;
+                if (G > 1) st_half(PT + (hn + kc) * Np + j, to_bits(pr), ecur, nonce);
+                __stcg(PR + (hn + kc) * P + j, pr);
                 const T z = pfma(-zq, pr, zs[c]);
                 zs[c] = z;
                 if (!DUAL) {
@@ -1335,8 +1495,12 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             }
             __syncwarp();
             // a full panel is applied after the next records: the rows it
-            // reads must have arrived before this CTA's record says so
-            if (G > 1 && kc + 1 == K) __threadfence();
+            // reads, and what the panel before it wrote, must have arrived
+            // before this CTA's record says so
+            if (kc + 1 == K) {
+                if (OV) wait_jobs();
+                if (G > 1) __threadfence();
+            }
             if (!DUAL) {
                 k = kc + 1;
                 publish_entering(vk, loc, flag);
@@ -1349,10 +1513,13 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             unsigned long long f = 0;
             if (row_warp) bad = form_col(q, e1.cta, e2.cta, 0, &f);
             // (as above; the row warps publish, the column warps wrote the rows)
-            if (kc + 1 == K) __syncthreads();
+            if (kc + 1 == K) {
+                if (OV) wait_jobs();
+                cta_sync();
+            }
             k = kc + 1;
             if (row_warp) {
-                update_rhs(kc, p, q, lane_value(f, kRhs1),
+                update_rhs(hn + kc, p, q, lane_value(f, kRhs1),
                            Divisor(lane_value(f, kDen2), lane_value(f, kRcp2)));
                 __syncwarp();
                 publish_leaving(nbland, bad);
@@ -1360,20 +1527,32 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             }
         } else if (row_warp) {
             const unsigned long long f = fetch(nullptr, 0, nullptr, -1, e2.cta, 0);
-            update_rhs(kc, p, q, lane_value(f, kNum2),
+            update_rhs(hn + kc, p, q, lane_value(f, kNum2),
                        Divisor(lane_value(f, kDen2), lane_value(f, kRcp2)));
         }
         k = kc + 1;
-        if (tid == 0) s_prow[kc] = p;
+        if (tid == 0) s_prow[hn + kc] = p;
     }
 
     // --------------------------------------------------------------- end --
-    if (status != ST_TIMEOUT && k > 0) {
+    if constexpr (OV) {
+        wait_jobs();
         // (every CTA takes this branch: the records decide, and they agree)
-        if (grid_sync(d->bar, err, G, spin_limit, &s_flag)) apply_panel(k);
+        if (status != ST_TIMEOUT && !group_barrier()) status = ST_TIMEOUT;
+        if (status != ST_TIMEOUT) {
+            if (jobs > 1) cur ^= 1, Tab = bufs[cur];
+            if (k > 0) {
+                for (int w = tid; w < nwords; w += B) out[w] = stay[w];
+                post(kJobInPlace, hn, k, !drop || nodrop);
+                wait_jobs();
+            }
+        }
+        post(kJobEnd, 0, 0, false);
+    } else if (status != ST_TIMEOUT && k > 0) {
+        if (group_barrier()) apply_panel(k);
         else status = ST_TIMEOUT;
     }
-    __syncthreads();
+    cta_sync();
     {
         T *z = Tab + (long long)m * P;
         for (int c = tid; c < W; c += B) z[c0 + c] = zs[c];
@@ -1386,7 +1565,9 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         d->deg = deg;
         d->last_p = last_p;
         d->last_q = last_q;
-        if (d->work) {
+        if (OV) {
+            if (status != ST_TIMEOUT) d->T = Tab, d->T2 = bufs[cur ^ 1];
+        } else if (d->work) {
             d->work[0] += upd;
             d->work[1] += left;
         }
@@ -1398,8 +1579,17 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     panel_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
                  unsigned nonce, long long limit_ns) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    panel_solve<T, DUAL, kPanelK>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce,
+    panel_solve<T, DUAL, kPanelK, false>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce,
                                   limit_ns, smem_raw);
+}
+
+template <bool DUAL>
+__global__ void __launch_bounds__(2 * kPanelThreads, 1)
+    panel_overlap_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
+                         unsigned nonce, long long limit_ns) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    panel_solve<double, DUAL, kPanelOverlapK, true>(d, gridDim.x, blockIdx.x, spin_limit, budget,
+                                                    drop, nonce, limit_ns, smem_raw);
 }
 
 // Many LPs in one launch.  items[] lists (lp, rank) pairs, the ranks of one LP
@@ -1425,10 +1615,10 @@ __global__ void __launch_bounds__(kPanelThreads, 2)
         const int2 w = items[it];
         LpDesc *d = descs + w.x;
         if (d->sense)
-            panel_solve<T, true, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
+            panel_solve<T, true, kPanelBatchK, false>(d, d->group, w.y, spin_limit, budget, drop, nonce,
                                                0, smem_raw);
         else
-            panel_solve<T, false, kPanelBatchK>(d, d->group, w.y, spin_limit, budget, drop, nonce,
+            panel_solve<T, false, kPanelBatchK, false>(d, d->group, w.y, spin_limit, budget, drop, nonce,
                                                 0, smem_raw);
     }
 }
@@ -1441,7 +1631,8 @@ unsigned next_nonce() {
 
 }  // namespace
 
-PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop) {
+PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop,
+                              bool overlap) {
     PivotShape sh;
     const int m = M - 1;
     // Default grid: every SM, on small LPs one CTA per two rows or 32 columns,
@@ -1450,14 +1641,14 @@ PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dua
     int G = ctas > 0 ? ctas : std::max((m + 1) / 2, (N + 31) / 32);
     G = std::min(G, std::min(sms, kPanelMaxCtas));
     G = std::max(1, std::min(G, N));
-    const size_t smem = panel_smem(prec, m, N, G, kPanelK);
+    const size_t smem = panel_smem(prec, m, N, G, kPanelK, overlap);
     sh.ctas = G;
-    sh.threads = kPanelThreads;
+    sh.threads = overlap ? 2 * kPanelThreads : kPanelThreads;
     sh.dual = dual;
     sh.drop = drop;
     sh.use_smem = 1;
     sh.smem_bytes = smem;
-    sh.pipe = smem <= kMaxDynSmem ? 4 : 0;
+    sh.pipe = smem > kMaxDynSmem ? 0 : overlap ? 5 : 4;
     return sh;
 }
 
@@ -1468,8 +1659,8 @@ size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K) 
     return tagged + (size_t)K * (size_t)P * esz;
 }
 
-size_t panel_smem(int prec, int m, int N, int G, int K) {
-    return panel_layout(m, N, G, prec == PREC_FP64 ? 8 : 4, prec == PREC_FP64 ? 2 : 4, K).total;
+size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap) {
+    return panel_layout(m, N, G, prec == PREC_FP64 ? 8 : 4, prec == PREC_FP64 ? 2 : 4, K, overlap).total;
 }
 
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
@@ -1478,10 +1669,12 @@ cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long lo
     unsigned nonce = next_nonce();
     long long limit_ns = sh.limit_ns;
     void *args[] = {&d_desc, &spin_limit, &budget, &drop, &nonce, &limit_ns};
-    const void *fn = prec == PREC_FP64 ? (sh.dual ? (const void *)panel_kernel<double, true>
-                                                  : (const void *)panel_kernel<double, false>)
-                                       : (sh.dual ? (const void *)panel_kernel<float, true>
-                                                  : (const void *)panel_kernel<float, false>);
+    const void *fn = sh.pipe == 5 ? (sh.dual ? (const void *)panel_overlap_kernel<true>
+                                             : (const void *)panel_overlap_kernel<false>)
+                     : prec == PREC_FP64 ? (sh.dual ? (const void *)panel_kernel<double, true>
+                                                    : (const void *)panel_kernel<double, false>)
+                                         : (sh.dual ? (const void *)panel_kernel<float, true>
+                                                    : (const void *)panel_kernel<float, false>);
     cudaError_t e = allow_dyn_smem(fn);
     if (e != cudaSuccess) return e;
     // A cooperative launch fails instead of running when the grid cannot be

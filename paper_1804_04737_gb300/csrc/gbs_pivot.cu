@@ -911,7 +911,7 @@ PivotShape choose_shape(int prec, int sense, int M, int N, long long P, int sms,
 
 cudaError_t launch_pivot(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s) {
-    if (sh.pipe == 4) return launch_panel(prec, d_desc, sh, spin_limit, budget, s);
+    if (sh.pipe >= 4) return launch_panel(prec, d_desc, sh, spin_limit, budget, s);
     if (sh.pipe) return launch_pivot_pipe(prec, d_desc, sh, spin_limit, budget, s);
     int W = sh.strip;
     void *args[] = {&d_desc, &W, &spin_limit, &budget};

@@ -86,3 +86,49 @@ def test_ratio_keys_out_of_range(e, sense):
         A, b, c = lpgen.dual_of(A, b, c)
         eps = {"eps_d": eps["eps_r"], "eps_p": eps["eps_p"], "eps_r": eps["eps_d"]}
     assert_same(Run(A, b, c, sense, zero_skip=2, **eps), _oracle(A, b, c, sense, **eps))
+
+
+# overlapped panels: from 2^20 tableau elements on (fewer than 450000 per CTA)
+@pytest.mark.parametrize("zero_skip", [0, 2])
+@pytest.mark.parametrize("sense", [MAX_LE, MIN_GE])
+@pytest.mark.parametrize("m,n,ctas", [(30, 36000, 0), (1500, 10, 0), (601, 1203, 0), (701, 800, 3),
+                                      (1023, 515, 152), (150, 8001, 20)])
+def test_overlapped_panels_bitwise(m, n, ctas, sense, zero_skip):
+    """Few rows or columns per CTA, uneven slices, few pivots (the copy of the
+    tableau still running when the pivots end) and many."""
+    m1, n1 = (m, n) if sense == MAX_LE else (n, m)
+    for A, b, c in (lpgen.dense_lp(m1, n1, seed=m + n), lpgen.paper_lp(m1, n1, seed=5)):
+        if sense == MIN_GE:
+            A, b, c = lpgen.dual_of(A, b, c)
+        kw = dict(max_iters=200)
+        assert_same(Run(A, b, c, sense, ctas=ctas, zero_skip=zero_skip, time_limit_s=60.0, **kw),
+                    _oracle(A, b, c, sense, **kw))
+
+
+@pytest.mark.parametrize("chunk", [1, 7, 8, 9, 16, 17, 24, 25])
+@pytest.mark.parametrize("kind", ["primal", "dual", "phase1"])
+def test_overlapped_calls_that_end_around_a_panel(chunk, kind):
+    """Calls of `chunk` pivots: ending with none, one or two panels begun, in
+    either buffer."""
+    m, n, sense = 600, 1200, MAX_LE
+    A, b, c = lpgen.dense_lp(m, n, seed=9)
+    if kind == "dual":
+        A, b, c = lpgen.dual_of(A, b, c)
+        sense = MIN_GE
+    if kind == "phase1":
+        A, b = lpgen.with_ge_rows(A, b, 0.02, seed=2)
+    calls = 6
+    h = capi.lp_create(capi.lp_options_default(max_iters=chunk))
+    try:
+        capi.lp_load(h, A, b, c, sense)
+        for k in range(calls):
+            capi.lp_solve(h)
+            _, st, it = capi.lp_result(h)
+            if st != capi.LP_ITER_LIMIT:
+                break
+        o = _oracle(A, b, c, sense, max_iters=chunk * (k + 1))
+        assert st == o.status and it == o.iters
+        assert np.array_equal(capi.lp_get_basis(h, A.shape[0]), o.basis)
+        assert np.array_equal(_bits(capi.lp_get_tableau(h, *A.shape)), _bits(o.T))
+    finally:
+        capi.lp_destroy(h)
