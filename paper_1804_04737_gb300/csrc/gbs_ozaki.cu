@@ -42,6 +42,16 @@
 // both with the tableau's signs (the dual form enters as -A, -b), rounded into
 // the FP32 tableau (basic columns set to exact unit vectors; the rhs column
 // and the objective row come from the reinversion's own FP64 values).
+// Nearly every slack is basic, and a basic slack's column is exactly zero in
+// X: the products run over the other columns only, in groups of four (16 bytes
+// of a tableau row), and a copy-bound kernel writes the unit columns.  The
+// exponents and digits of the columns that remain, and so every bit written,
+// are those of the products over all columns.  At 8192 x 8192 with 50 to 334
+// structural basics the second product takes 0.88 ms and the unit columns
+// 0.05, against 1.30 over all columns; with one MMA in six of the 334's it
+// takes as long, so its epilogue bounds it: by switching parts off, about 0.23
+// ms each are FP64 operations (two a value) and the sums' first steps, 0.14 the
+// reads of A.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -242,16 +252,18 @@ struct SrcGather {  // sg * A[rows[i]][cols[k]] (A row-major with n columns)
     double sg;
     __device__ double at(int i, int k) const { return sg * A[(long long)rows[i] * n + cols[k]]; }
 };
-struct SrcRefreshB {  // row r: [sg A_l | e_l | sg b_l], l = R[r]
+struct SrcRefreshB {  // row r: the groups' columns of [sg A_l | e_l], then sg b_l, l = R[r]
     const double *A, *b;
-    const int *R;
-    int n, m;
+    const int *R, *grp;
+    int n, ng;  // ng groups
     double sg;
-    __device__ double at(int r, int j) const {
+    __device__ double at(int r, int e) const {
         const int l = R[r];
+        if (e >= 4 * ng) return sg * b[l];
+        const int g = grp[e >> 2], j = 4 * g + (e & 3);
+        if (g < 0) return 0.0;
         if (j < n) return sg * A[(long long)l * n + j];
-        if (j < n + m) return (j - n == l) ? 1.0 : 0.0;
-        return sg * b[l];
+        return (j - n == l) ? 1.0 : 0.0;
     }
 };
 
@@ -284,18 +296,30 @@ __global__ void oz_kexpA_kernel(Src src, int M, int K, int *kA) {
     }
 }
 
-// eB_k: largest exponent of row k of B (K x N), one warp per k; then shift_k.
-template <class Src>
-__global__ void oz_kexpB_kernel(Src src, int K, int N, const int *kA, int *shift) {
-    const int k = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (k >= K) return;
+// eB_k: largest exponent of row k of B (K x N), one block of 256 per k
+// (kWide) or one warp; then shift_k.  Long rows get a block: with one warp, 334
+// rows of 16385 took 136 us, most of the chip idle.
+template <class Src, bool kWide>
+__global__ void __launch_bounds__(256) oz_kexpB_kernel(Src src, int K, int N, const int *kA, int *shift) {
+    __shared__ int red[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = kWide ? (int)blockIdx.x : (int)(blockIdx.x * 8 + warp);
     int mx = kNoExp;
-    for (int j = lane; j < N; j += 32) {
-        const int ex = exp_of(src.at(k, j));
-        if (ex) mx = max(mx, ex);
+    if (k < K) {
+#pragma unroll 4
+        for (int j = kWide ? threadIdx.x : lane; j < N; j += kWide ? 256 : 32) {
+            const int ex = exp_of(src.at(k, j));
+            if (ex) mx = max(mx, ex);
+        }
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) shift[k] = (mx != kNoExp && kA[k] != 0) ? (mx - kA[k]) >> 1 : 0;
+    if (kWide) {
+        if (lane == 0) red[warp] = mx;
+        __syncthreads();
+        for (int w = 0; w < 8; ++w) mx = max(mx, red[w]);
+    }
+    if (k < K && (kWide ? threadIdx.x : lane) == 0)
+        shift[k] = (mx != kNoExp && kA[k] != 0) ? (mx - kA[k]) >> 1 : 0;
 }
 
 // Largest shifted exponent of each row i < M of A over k < K (kNoExp: none).
@@ -419,18 +443,19 @@ struct OzParams {
     // digit planes with a nonzero digit, per 128-row block of A and per
     // 64-column block of B (bit p: plane p; plane 0 always set)
     const int *amask, *bmask;
-    int mode;  // 0: C = A B (FP64, rows < M, cols < N); 1: refresh rows into the FP32 tableau
+    // mode 0: C = A B (FP64, rows < M, cols < N); mode 1: refresh rows into the FP32 tableau
     double *C;
     long long ldc;
-    // mode 1: output row r is tableau row rowmap[r], constraint rowk[r]; the
-    // value written is sg [A_k | e_k](j) - (A B)_rj for j < N, with the
-    // basic columns set to unit vectors (basic_row[j]: the row where column j
-    // is basic, or -1)
+    // mode 1: output row r is tableau row rowmap[r], constraint rowk[r], and
+    // columns 4 g .. 4 g + 3 of the product are columns 4 grp[g] .. + 3 of the
+    // tableau (grp[g] < 0: none); the value written is sg [A_k | e_k](j) -
+    // (A B)_rj for tableau columns j < cols, with the basic columns set to unit
+    // vectors (basic_row[j]: the row where column j is basic, or -1)
     float *T32;
     long long P;
-    const int *rowmap, *rowk, *basic_row;
+    const int *rowmap, *rowk, *basic_row, *grp;
     const double *Aorig;
-    int n, m;
+    int n, cols;
     double sg;
     int *err;
     unsigned long long *mmas;  // += the tcgen05.mma instructions issued (128 x 64 x 16 each)
@@ -474,12 +499,35 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// Four doubles at p + j (32-byte aligned), zeros where j is outside [0, n).
+__device__ __forceinline__ void ldg4(const double *p, int j, int n, double *x) {
+    x[0] = x[1] = x[2] = x[3] = 0.0;
+    if ((unsigned)j < (unsigned)n)
+        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                     : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3])
+                     : "l"(p + j));
+}
+// x rounded to the nearest float, ties to even, by integer operations where the
+// result is a normal float: the conversion instruction shares the FP64 pipe.
+__device__ __forceinline__ float round_f32(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const unsigned e = (unsigned)(u >> 52) & 0x7ffu;
+    if (e - 897u < 253u) {  // 2^-126 <= |x| < 2^127
+        const unsigned long long a = u & 0x7fffffffffffffffull;
+        const unsigned long long r = a + 0x0fffffffull + ((a >> 29) & 1ull);
+        return __uint_as_float(((unsigned)(r >> 29) - (896u << 23)) | ((unsigned)(u >> 32) & 0x80000000u));
+    }
+    return __double2float_rn(x);
+}
+
+// (one instance per mode: the other's epilogue would cost it registers)
+template <int MODE>
 __global__ void __launch_bounds__(kOzThreads, 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const OzParams p) {
     extern __shared__ unsigned char oz_smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ int s_colexp[kOzBN], s_brow[kOzBN];
+    __shared__ int s_colexp[kOzBN], s_brow[kOzBN], s_gj[kOzBN / 4];
     const uint32_t raw = su32(oz_smem);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t sB = base;                                  // [stages][S][64][128 B]
@@ -674,7 +722,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             if (et < kOzBN) {
                 const int col = n0 + et;
                 s_colexp[et] = col < p.N ? p.colexp[col] : kNoExp;
-                if (p.mode == 1) s_brow[et] = col < p.N - 1 ? p.basic_row[col] : -1;
+                if (MODE == 1) {
+                    const int gr = p.grp[col >> 2], j = 4 * gr + (col & 3);
+                    s_brow[et] = gr >= 0 && j < p.cols ? p.basic_row[j] : -1;
+                    if ((et & 3) == 0) s_gj[et >> 2] = j;
+                }
             }
             const int Er = r < p.M ? p.rowexp[r] : kNoExp;
             uint32_t gm = 0u;
@@ -689,15 +741,27 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             int ti = 0, kr = 0;
             const double *arow = p.Aorig;
             double av[8];
-            auto orig = [&](double (&x)[8], int j0) {
+            // (rows of A on 32 bytes, as the groups are: one read per group
+            // instead of four, and the rounding by integers: 1.02 -> 0.88 ms)
+            const bool quads = ((p.n & 3) | (int)((unsigned long long)p.Aorig & 31)) == 0;
+            auto orig = [&](double (&x)[8], int ja, int jb) {
+                if (quads) {
+                    ldg4(arow, ja, p.n, x);
+                    ldg4(arow, jb, p.n, x + 4);
+                    return;
+                }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] = j0 + j < p.n ? __ldg(arow + j0 + j) : 0.0;
+                for (int j = 0; j < 8; ++j) {
+                    const int jt = (j < 4 ? ja : jb) + (j & 3);
+                    x[j] = (unsigned)jt < (unsigned)p.n ? __ldg(arow + jt) : 0.0;
+                }
             };
-            if (p.mode == 1 && r < p.M) {
+            if (MODE == 1 && r < p.M) {
+                const int2 gq = __ldg(reinterpret_cast<const int2 *>(p.grp) + (n0 >> 3) + 2 * hsel);
                 ti = p.rowmap[r];
                 kr = p.rowk[r];
                 arow += (long long)kr * p.n;
-                orig(av, n0 + hsel * 16);
+                orig(av, 4 * gq.x, 4 * gq.y);
             }
             for (int c = 0; c < nch && ok; ++c) {
                 // all the epilogue warps leave together or go on together
@@ -753,7 +817,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     // tensor-memory lane holds): one contiguous row segment per
                     // thread, read (C, or the original row of A) and written with
                     // independent accesses, no shared-memory transposition.
-                    if (p.mode == 0) {
+                    if constexpr (MODE == 0) {
                         if (r < p.M) {
                             double *crow = p.C + (long long)r * p.ldc + j0;
 #pragma unroll
@@ -769,9 +833,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                         const long long sgbit = p.sg < 0.0 ? (long long)kSign : 0ll;
                         float *trow = p.T32 + (long long)ti * p.P;
                         double aw[8];
-                        orig(aw, j0 + 8);
+                        const int *gj = s_gj + (cb >> 2);
+                        orig(aw, gj[2], gj[3]);
                         auto refreshed = [&](int j, double aj) {
-                            const int col = j0 + j, br = s_brow[cb + j];
+                            const int col = gj[j >> 2] + (j & 3), br = s_brow[cb + j];
                             if (br >= 0) return br == ti ? 1.0f : 0.0f;
                             const int Fc = s_colexp[cb + j];
                             double v = 0.0;
@@ -780,10 +845,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                             // sg A_kj by its sign bit (no FP64 multiply)
                             const double d = col < p.n ? __longlong_as_double(__double_as_longlong(aj) ^ sgbit)
                                                        : (col - p.n == kr ? 1.0 : 0.0);
-                            return __double2float_rn(d - v);
+                            return round_f32(d - v);
                         };
                         // (the rhs column comes from the reinversion; the rows
-                        // are 128-byte aligned, the columns here 64)
+                        // are 128-byte aligned, the groups 16)
 #pragma unroll
                         for (int j = 0; j < 16; j += 4) {
                             float4 o;
@@ -791,12 +856,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                             o.y = refreshed(j + 1, j < 8 ? av[(j & 7) + 1] : aw[(j & 7) + 1]);
                             o.z = refreshed(j + 2, j < 8 ? av[(j & 7) + 2] : aw[(j & 7) + 2]);
                             o.w = refreshed(j + 3, j < 8 ? av[(j & 7) + 3] : aw[(j & 7) + 3]);
-                            if (j0 + j + 3 < p.N - 1) {
-                                *reinterpret_cast<float4 *>(trow + j0 + j) = o;
+                            const int jt = gj[j >> 2];
+                            if (jt < 0) continue;
+                            if (jt + 3 < p.cols) {
+                                *reinterpret_cast<float4 *>(trow + jt) = o;
                             } else {
-                                if (j0 + j < p.N - 1) trow[j0 + j] = o.x;
-                                if (j0 + j + 1 < p.N - 1) trow[j0 + j + 1] = o.y;
-                                if (j0 + j + 2 < p.N - 1) trow[j0 + j + 2] = o.z;
+                                if (jt < p.cols) trow[jt] = o.x;
+                                if (jt + 1 < p.cols) trow[jt + 1] = o.y;
+                                if (jt + 2 < p.cols) trow[jt + 2] = o.z;
                             }
                         }
                     }
@@ -890,10 +957,11 @@ cudaError_t oz_reserve(OzWork &w, int M, int N, int K) {
 
 // Digits of A (M x K from srcA) and B (K x N from srcB), then the product.
 // The workspace must already hold this size (oz_reserve): growing it here
-// could free a buffer that queued work still reads.
-template <class SA, class SB>
+// could free a buffer that queued work still reads.  (B's first Nexp columns,
+// if more than N, take part in the inner balancing only.)
+template <int MODE, class SA, class SB>
 cudaError_t oz_product(SA srcA, SB srcB, int M, int N, int K, OzParams p, OzWork &w, int sms,
-                       cudaStream_t s) {
+                       cudaStream_t s, int Nexp = 0) {
     const int Mp = round_up(std::max(M, 1), kOzBM), Np = round_up(std::max(N, 1), kOzBN),
               Kp = round_up(std::max(K, 1), kOzBK);
     cudaError_t e;
@@ -909,7 +977,9 @@ cudaError_t oz_product(SA srcA, SB srcB, int M, int N, int K, OzParams p, OzWork
     if (K > 0) {
         if ((e = cudaMemsetAsync(kA, 0, sizeof(int) * (size_t)K, s)) != cudaSuccess) return e;
         oz_kexpA_kernel<SA><<<dim3((K + 31) / 32, (M + 63) / 64), 256, 0, s>>>(srcA, M, K, kA);
-        oz_kexpB_kernel<SB><<<(K + 7) / 8, 256, 0, s>>>(srcB, K, N, kA, shift);
+        const int Nb = std::max(N, Nexp);
+        if (Nb >= 2048) oz_kexpB_kernel<SB, true><<<K, 256, 0, s>>>(srcB, K, Nb, kA, shift);
+        else oz_kexpB_kernel<SB, false><<<(K + 7) / 8, 256, 0, s>>>(srcB, K, Nb, kA, shift);
     }
     oz_rowexp_kernel<SA><<<(M + 7) / 8, 256, 0, s>>>(srcA, M, K, shift, w.rowexp);
     oz_colexp_kernel<SB><<<(N + 255) / 256, 256, 0, s>>>(srcB, K, N, shift, w.colexp);
@@ -939,19 +1009,19 @@ cudaError_t oz_product(SA srcA, SB srcB, int M, int N, int K, OzParams p, OzWork
     p.mmas = w.mmas;
     if ((e = cudaMemsetAsync(p.err, 0, sizeof(int), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(p.mmas, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    if (p.mode == 1 && Kp > kOzChunkKB * kOzBK) return cudaErrorInvalidValue;  // one chunk only
-    if ((e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (MODE == 1 && Kp > kOzChunkKB * kOzBK) return cudaErrorInvalidValue;  // one chunk only
+    if ((e = cudaFuncSetAttribute(oz_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kOzSmem)) != cudaSuccess)
         return e;
     const int tiles = (Mp / kOzBM) * (Np / kOzBN);
-    oz_gemm_kernel<<<std::min(tiles, sms), kOzThreads, kOzSmem, s>>>(ma, mb, p);
+    oz_gemm_kernel<MODE><<<std::min(tiles, sms), kOzThreads, kOzSmem, s>>>(ma, mb, p);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 void oz_work_free(OzWork &w) {
-    void *ps[] = {w.asl, w.bsl, w.rowexp, w.colexp, w.kx, w.pmask, w.X, w.Ainv, w.Z, w.basic_row, w.L, w.Lrow, w.err,
+    void *ps[] = {w.asl, w.bsl, w.rowexp, w.colexp, w.kx, w.pmask, w.X, w.Ainv, w.Z, w.basic_row, w.L, w.Lrow, w.grp, w.err,
                   w.mmas};
     for (void *q : ps)
         if (q) cudaFree(q);
@@ -964,12 +1034,11 @@ cudaError_t oz_dgemm(const double *A, long long lda, const double *B, long long 
     cudaError_t e = oz_reserve(w, M, N, K);
     if (e != cudaSuccess) return e;
     OzParams p{};
-    p.mode = 0;
     p.C = C;
     p.ldc = ldc;
     p.err = d_err;
     p.spin_limit = spin_limit;
-    return oz_product(SrcDense{A, lda}, SrcDense{B, ldb}, M, N, K, p, w, sms, s);
+    return oz_product<0>(SrcDense{A, lda}, SrcDense{B, ldb}, M, N, K, p, w, sms, s);
 }
 
 namespace {
@@ -1022,36 +1091,99 @@ __global__ void __launch_bounds__(1024) oz_llist_kernel(const int *__restrict__ 
     }
 }
 
+// grp = the groups of four tableau columns (of the first `cols`) that are not
+// all basic slacks, ascending, then -1 up to `cap` (one CTA of 1024 threads).
+__global__ void __launch_bounds__(1024) oz_groups_kernel(const int *__restrict__ basic_row, int n,
+                                                         int cols, int cap, int *__restrict__ grp) {
+    __shared__ int scan[1024];
+    const int tid = threadIdx.x, B = blockDim.x, total = (cols + 3) / 4;
+    const int chunk = (total + B - 1) / B;
+    const int g0 = min(total, tid * chunk), g1 = min(total, g0 + chunk);
+    auto kept = [&](int g) {
+        if (4 * g < n) return true;
+        bool some = false;
+        for (int j = 4 * g; j < min(cols, 4 * g + 4); ++j) some |= basic_row[j] < 0;
+        return some;
+    };
+    int cnt = 0;
+    for (int g = g0; g < g1; ++g) cnt += kept(g);
+    scan[tid] = cnt;
+    __syncthreads();
+    for (int o = 1; o < B; o <<= 1) {
+        const int a = tid >= o ? scan[tid - o] : 0;
+        __syncthreads();
+        scan[tid] += a;
+        __syncthreads();
+    }
+    int k = scan[tid] - cnt;
+    for (int g = g0; g < g1; ++g)
+        if (kept(g) && k < cap) grp[k++] = g;
+    for (int e = scan[B - 1] + tid; e < cap; e += B) grp[e] = -1;
+}
+
+// The other groups' columns, in all m rows: unit vectors.
+__global__ void __launch_bounds__(256) oz_unit_kernel(const int *__restrict__ basic_row, int m, int n,
+                                                      int cols, float *__restrict__ T32, long long P) {
+    const int g = (n + 3) / 4 + blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = 4 * g;
+    if (j >= cols) return;
+    int br[4];
+    bool all = true;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        br[u] = j + u < cols ? basic_row[j + u] : 0;
+        all &= br[u] >= 0;
+    }
+    if (!all) return;
+    const bool whole = j + 3 < cols;
+#pragma unroll 4
+    for (int i = blockIdx.y; i < m; i += gridDim.y) {
+        float *at = T32 + (long long)i * P + j;
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = br[u] == i ? 1.0f : 0.0f;
+        if (whole) *reinterpret_cast<float4 *>(at) = make_float4(v[0], v[1], v[2], v[3]);
+        else
+            for (int u = 0; u < 4 && j + u < cols; ++u) at[u] = v[u];
+    }
+}
+
 // The rows of the structural basics: tableau row basic_row[S[k]] = X[k] in
-// FP32, basic columns as unit vectors, every column but the rhs.
-__global__ void oz_xrows_kernel(const double *__restrict__ X, int N, int ns, const int *__restrict__ S,
-                                const int *__restrict__ basic_row, float *__restrict__ T32, long long P) {
-    const long long total = (long long)ns * (N - 1);
+// FP32 at the groups' columns, basic columns as unit vectors.
+__global__ void oz_xrows_kernel(const double *__restrict__ X, int ldx, int ns, const int *__restrict__ S,
+                                const int *__restrict__ basic_row, const int *__restrict__ grp, int ng,
+                                int cols, float *__restrict__ T32, long long P) {
+    const long long total = (long long)ns * ng * 4;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(e / (N - 1)), j = (int)(e - (long long)k * (N - 1));
+        const int k = (int)(e / (4 * ng)), c = (int)(e - (long long)k * (4 * ng));
+        const int g = grp[c >> 2], j = 4 * g + (c & 3);
+        if (g < 0 || j >= cols) continue;
         const int ti = basic_row[S[k]], br = basic_row[j];
-        T32[(long long)ti * P + j] = br >= 0 ? (br == ti ? 1.0f : 0.0f) : (float)X[(long long)k * N + j];
+        T32[(long long)ti * P + j] = br >= 0 ? (br == ti ? 1.0f : 0.0f) : (float)X[(long long)k * ldx + c];
     }
 }
 
 // The rows of the slack basics from Z = A_LS X (when the product took more
 // than one K chunk): sg [A_l | e_l](j) - Z[r][j].
-__global__ void oz_yrows_kernel(const double *__restrict__ Z, int N, int mL, const int *__restrict__ L,
+__global__ void oz_yrows_kernel(const double *__restrict__ Z, int mL, const int *__restrict__ L,
                                 const int *__restrict__ Lrow, const double *__restrict__ A, int n,
-                                double sg, const int *__restrict__ basic_row, float *__restrict__ T32,
+                                double sg, const int *__restrict__ basic_row,
+                                const int *__restrict__ grp, int ng, int cols, float *__restrict__ T32,
                                 long long P) {
-    const long long total = (long long)mL * (N - 1);
+    const long long total = (long long)mL * ng * 4;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(e / (N - 1)), j = (int)(e - (long long)r * (N - 1));
+        const int r = (int)(e / (4 * ng)), c = (int)(e - (long long)r * (4 * ng));
+        const int g = grp[c >> 2], j = 4 * g + (c & 3);
+        if (g < 0 || j >= cols) continue;
         const int ti = Lrow[r], l = L[r], br = basic_row[j];
         float v;
         if (br >= 0) {
             v = br == ti ? 1.0f : 0.0f;
         } else {
             const double d = j < n ? sg * A[(long long)l * n + j] : (j - n == l ? 1.0 : 0.0);
-            v = (float)(d - Z[(long long)r * N + j]);
+            v = (float)(d - Z[e]);
         }
         T32[(long long)ti * P + j] = v;
     }
@@ -1068,43 +1200,52 @@ cudaError_t oz_refresh_body(const double *A, const double *b, int sense, int m, 
                             long long P, OzWork &w, int sms, long long spin_limit,
                             cudaStream_t s) {
     const double sg = sense == 0 ? 1.0 : -1.0;
-    const int N = n + m + 1, mL = m - ns;
+    const int cols = n + m, mL = m - ns;
+    // groups of four columns that hold a structural or (ns of them) nonbasic
+    // slack, and the columns of X: theirs and the rhs
+    const int ng = std::min((cols + 3) / 4, (n + 3) / 4 + ns), N = 4 * ng, Nx = N + 1;
+    const int gcap = round_up(Nx, kOzBN) / 4;
     const bool one_chunk = round_up(std::max(ns, 1), kOzBK) <= kOzChunkKB * kOzBK;
     cudaError_t e;
     // every buffer at its final size before any work is queued
     if ((e = grow_buf(&w.basic_row, &w.cap_basic, (size_t)(n + m))) != cudaSuccess) return e;
     if ((e = grow_buf(&w.L, &w.cap_L, (size_t)m)) != cudaSuccess) return e;
     if ((e = grow_buf(&w.Lrow, &w.cap_Lrow, (size_t)m)) != cudaSuccess) return e;
-    if ((e = grow_buf(&w.X, &w.cap_X, (size_t)ns * N)) != cudaSuccess) return e;
+    if ((e = grow_buf(&w.X, &w.cap_X, (size_t)ns * Nx)) != cudaSuccess) return e;
     if ((e = grow_buf(&w.Ainv, &w.cap_Ainv, (size_t)ns * ns)) != cudaSuccess) return e;
     if (!one_chunk && (e = grow_buf(&w.Z, &w.cap_Z, (size_t)mL * N)) != cudaSuccess) return e;
-    if ((e = oz_reserve(w, ns, N, ns)) != cudaSuccess) return e;
+    if ((e = grow_buf(&w.grp, &w.cap_grp, (size_t)gcap)) != cudaSuccess) return e;
+    if ((e = oz_reserve(w, ns, Nx, ns)) != cudaSuccess) return e;
     if ((e = oz_reserve(w, mL, N, ns)) != cudaSuccess) return e;
 
     if ((e = cudaMemsetAsync(w.basic_row, 0xff, sizeof(int) * (size_t)(n + m), s)) != cudaSuccess)
         return e;
     oz_basic_kernel<<<(m + 255) / 256, 256, 0, s>>>(basis, m, w.basic_row);
     oz_llist_kernel<<<1, 1024, 0, s>>>(w.basic_row, m, n, w.L, w.Lrow);
+    oz_groups_kernel<<<1, 1024, 0, s>>>(w.basic_row, n, cols, gcap, w.grp);
+    {
+        const int gs = std::max(1, (cols + 3) / 4 - (n + 3) / 4), bx = (gs + 255) / 256;
+        oz_unit_kernel<<<dim3(bx, std::max(1, std::min(m, 16 * sms / bx))), 256, 0, s>>>(
+            w.basic_row, m, n, cols, T32, P);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (ns > 0) {
         oz_ainv_kernel<<<grid_for((long long)ns * ns), 256, 0, s>>>(rb.W, rb.Wp, ns, rb.pivrow, w.Ainv);
         OzParams p{};
-        p.mode = 0;
         p.C = w.X;
-        p.ldc = N;
+        p.ldc = Nx;
         p.spin_limit = spin_limit;
-        e = oz_product(SrcDense{w.Ainv, ns}, SrcRefreshB{A, b, rb.R, n, m, sg}, ns, N, ns, p, w,
-                       sms, s);
+        e = oz_product<0>(SrcDense{w.Ainv, ns}, SrcRefreshB{A, b, rb.R, w.grp, n, ng, sg}, ns, Nx, ns,
+                       p, w, sms, s);
         if (e != cudaSuccess) return e;
-        oz_xrows_kernel<<<grid_for((long long)ns * (N - 1)), 256, 0, s>>>(w.X, N, ns, rb.S,
-                                                                           w.basic_row, T32, P);
+        oz_xrows_kernel<<<grid_for((long long)ns * N), 256, 0, s>>>(w.X, Nx, ns, rb.S, w.basic_row, w.grp,
+                                                                     ng, cols, T32, P);
     }
     if (mL > 0) {
         OzParams p{};
         p.spin_limit = spin_limit;
         const SrcGather a2{A, n, w.L, rb.S, sg};
         if (one_chunk) {
-            p.mode = 1;
             p.T32 = T32;
             p.P = P;
             p.rowmap = w.Lrow;
@@ -1112,17 +1253,17 @@ cudaError_t oz_refresh_body(const double *A, const double *b, int sense, int m, 
             p.basic_row = w.basic_row;
             p.Aorig = A;
             p.n = n;
-            p.m = m;
+            p.grp = w.grp;
+            p.cols = cols;
             p.sg = sg;
-            e = oz_product(a2, SrcDense{w.X, N}, mL, N, ns, p, w, sms, s);
+            e = oz_product<1>(a2, SrcDense{w.X, Nx}, mL, N, ns, p, w, sms, s, Nx);
         } else {
-            p.mode = 0;
             p.C = w.Z;
             p.ldc = N;
-            e = oz_product(a2, SrcDense{w.X, N}, mL, N, ns, p, w, sms, s);
+            e = oz_product<0>(a2, SrcDense{w.X, Nx}, mL, N, ns, p, w, sms, s, Nx);
             if (e == cudaSuccess)
-                oz_yrows_kernel<<<grid_for((long long)mL * (N - 1)), 256, 0, s>>>(
-                    w.Z, N, mL, w.L, w.Lrow, A, n, sg, w.basic_row, T32, P);
+                oz_yrows_kernel<<<grid_for((long long)mL * N), 256, 0, s>>>(
+                    w.Z, mL, w.L, w.Lrow, A, n, sg, w.basic_row, w.grp, ng, cols, T32, P);
         }
         if (e != cudaSuccess) return e;
     }
