@@ -11,18 +11,18 @@ every k in {50, 200} pivots, with its objective error against the FP64
 oracle.
 
 `value` is pivots per second over the whole job, device-timed with CUDA
-events on the library's stream, inputs resident in HBM.  The tableau (1.07 GB,
-two buffers) is larger than L2, so nothing survives in L2 from one step to
+events on the library's stream, inputs resident in HBM.  The tableau (1.07 GB)
+is larger than L2, so nothing survives in L2 from one step to
 the next.  `e2e` is the same metric through the C ABI with host buffers:
 lp_load from pinned host memory, lp_solve, lp_result into pinned host memory,
 wall clock.  `roofline` is that of the pivot kernel (one launch per solve):
 the FP64 FMA rate of the fmas it executes (one per updated tableau element
-and pivot; the two-pivot primal kernel leaves in place the column vectors
-whose entries in both pivot rows of a pass are zero, and counts what it
-updates) and the DRAM bytes it moves (from an ncu record of the same
-launch), the larger fraction leading; pivot-equivalent GB/s (2 x tableau
-bytes per pivot) is reported beside them, not as a bound: two pivots share
-one pass over the tableau, and vectors left in place are not moved.
+and pivot; the panel kernel leaves out the columns that stay basic through a
+panel of pivots, and counts what it updates) and the DRAM bytes it moves
+(from an ncu record of the same launch), the larger fraction leading;
+pivot-equivalent GB/s (2 x tableau bytes per pivot) is reported beside them,
+not as a bound: the pivots of a panel share one pass over the tableau, and
+columns left out are not moved.
 
 Other workloads (--workload): lp2048set (2048^2 primal and dual form,
 512 x 4096, 4096 x 512), paperset (the same shapes from the paper's random
@@ -43,7 +43,7 @@ if ROOT not in sys.path:
 MAX_LE, MIN_GE = 0, 1
 HBM_NOMINAL_GBS = 7900.0          # GB300 HBM3e nominal
 FP64_DFMA_PER_CLK_SM = 2          # GB300 FP64: 1.25 TFLOP/s nominal = 2 DFMA per clock per SM
-KERNEL_SRC = os.path.join(ROOT, "paper_1804_04737_gb300", "csrc", "gbs_pipe.cu")
+KERNEL_SRC = os.path.join(ROOT, "paper_1804_04737_gb300", "csrc", "gbs_panel.cu")
 
 WORKLOADS = {
     "lp8192": ("dense LP 8192x8192 (tableau 8193x16385, 1.07 GB FP64), primal form, FP64, Dantzig "
@@ -79,8 +79,7 @@ def bench_config(name, world):
     cfg = {"workload": WORKLOADS[name], "seed": 0,
            "parallelism": "replicas" if world > 1 else "single GPU"}
     if name == "lp8192":
-        cfg.update({"m": 8192, "n": 8192, "l2": "inputs larger than L2 (1.07 GB tableau, "
-                                                 "two buffers)"})
+        cfg.update({"m": 8192, "n": 8192, "l2": "inputs larger than L2 (1.07 GB tableau)"})
     else:
         cfg["l2"] = "flushed between steps (256 MiB write), outside the step events"
     return cfg
@@ -136,27 +135,26 @@ def device_fp64_peak(index):
     return tf, "derived: %d FP64 FMA/clk/SM x %d SMs x %.0f MHz" % (FP64_DFMA_PER_CLK_SM, sms, mhz)
 
 
-# The kernel each LP runs on (default options): primal LPs below 2^19 tableau
-# elements on the pipelined primal kernel in place, larger ones on the
-# two-pivots-per-pass kernel (double-buffered), the dual form on the
-# two-pivots-per-pass dual simplex kernel (double-buffered).
-INPLACE_KERNEL = "pivot_pipe_kernel<double> (in place)"
-BLOCK_KERNEL = "pivot_block_kernel<double> (two pivots per pass)"
-DUAL_KERNEL = "pivot_block_dual_kernel<double> (dual simplex, two pivots per pass)"
-# DRAM records (ncu) per kernel and workload; the in-place kernel runs no LP of
-# these sets, so it has none
+# The kernel each LP runs on (default options): the panel kernel, with the
+# panels under the selection of the next pivots from 2^20 tableau elements up to
+# 450000 per SM.
+PANEL_KERNELS = {
+    (MAX_LE, False): "panel_kernel<double, 0> (panels of 16 pivots, in turn with the selection)",
+    (MIN_GE, False): "panel_kernel<double, 1> (dual simplex, panels of 16 pivots, in turn with the selection)",
+    (MAX_LE, True): "panel_overlap_kernel<0> (panels of 8 pivots under the selection)",
+    (MIN_GE, True): "panel_overlap_kernel<1> (dual simplex, panels of 8 pivots under the selection)",
+}
+# DRAM records (ncu) per kernel and workload
 TRAFFIC_FILES = {
-    ("lp8192", BLOCK_KERNEL): "pivot_block_kernel_fp64_8192_traffic.txt",
-    ("lp2048set", BLOCK_KERNEL): "pivot_block_kernel_fp64_traffic.txt",
-    ("lp2048set", DUAL_KERNEL): "pivot_block_dual_kernel_fp64_traffic.txt",
+    ("lp8192", PANEL_KERNELS[MAX_LE, False]): "panel_kernel_fp64_8192_traffic.txt",
+    ("lp2048set", PANEL_KERNELS[MAX_LE, True]): "panel_overlap_kernel_fp64_traffic.txt",
+    ("lp2048set", PANEL_KERNELS[MIN_GE, True]): "panel_overlap_dual_kernel_fp64_traffic.txt",
 }
 
 
-def kernel_of(m, n, sense):
-    if sense != MAX_LE:
-        return DUAL_KERNEL
-    pitch = (n + m + 1 + 31) // 32 * 32
-    return INPLACE_KERNEL if (m + 1) * pitch < 2 ** 19 else BLOCK_KERNEL
+def kernel_of(m, n, sense, sms):
+    elems = (m + 1) * ((n + m + 1 + 31) // 32 * 32)
+    return PANEL_KERNELS[sense, 2 ** 20 <= elems < 450000 * sms]
 
 
 def kernel_traffic(wname, kernel):
@@ -729,6 +727,7 @@ def run_lpset(args, capi, torch, rank, world, local, dist):
     torch.cuda.synchronize()
     if dist:
         dist.barrier()
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
     step_ms, pivots, kernel_ms, alg_bytes = [], 0, 0.0, 0.0
     # name -> [launches, ms, algorithmic bytes, pivots, flops, executed flops,
     #          constraint-row entries updated, left in place]
@@ -745,7 +744,7 @@ def run_lpset(args, capi, torch, rank, world, local, dist):
                 kernel_ms += kms
                 by = it * tableau_bytes(m, n)
                 alg_bytes += by
-                rec = per_kernel.setdefault(kernel_of(m, n, sense),
+                rec = per_kernel.setdefault(kernel_of(m, n, sense, sms),
                                             [0, 0.0, 0.0, 0, 0.0, 0.0, 0, 0])
                 rec[0] += 1
                 rec[1] += kms
@@ -753,7 +752,7 @@ def run_lpset(args, capi, torch, rank, world, local, dist):
                 rec[3] += it
                 rec[4] += it * tableau_flops(m, n)
                 # the fmas executed: the updated constraint-row entries (the
-                # two-pivot primal kernel counts them) and the objective row
+                # panel kernel counts them) and the objective row
                 pitch = (n + m + 1 + 31) // 32 * 32
                 rec[5] += 2 * (upd + it * pitch) if upd + kept else it * tableau_flops(m, n)
                 rec[6] += upd
@@ -807,8 +806,8 @@ def run_lpset(args, capi, torch, rank, world, local, dist):
         CUDA-event duration: FP64 FMA (the fmas it executes: one per updated
         element and pivot) and the DRAM bytes it moves (ncu record); the
         larger fraction leads.  Pivot-equivalent GB/s (2 x tableau bytes per
-        pivot) is reported too; it is not a bound, since two pivots share one
-        pass over the tableau and vectors left in place are not moved."""
+        pivot) is reported too; it is not a bound, since the pivots of a panel
+        share one pass over the tableau and columns left out are not moved."""
         launches, ms, by, piv, flops, xflops, upd, kept = per_kernel[name]
         sec = ms * 1e-3
         traffic = kernel_traffic(wname, name)

@@ -136,12 +136,17 @@ typedef struct {
                                 1 = auto (default): the panel kernel, for the
                                     primal and the dual rule: pivots are
                                     selected on rows and columns formed on
-                                    demand and applied to the tableau, in
-                                    place, up to 16 at a time; where it cannot
-                                    take the LP (its workspace or its shared
-                                    memory does not fit) or n > 4 m from 2^20
-                                    tableau elements on, 2 below 2^19 elements
-                                    ((m+1) x row pitch), else 4 (2 when the
+                                    demand and applied to the tableau up to 16
+                                    at a time in place or, in FP64 from 2^20
+                                    tableau elements ((m+1) x row pitch) up to
+                                    450000 per CTA, up to 8 at a time into a
+                                    second buffer (in place where it cannot be
+                                    allocated) while the next are selected;
+                                    where the panel kernel cannot take the LP
+                                    (its workspace or its shared memory does
+                                    not fit), and with n > 4 m from 2^20
+                                    elements on in FP32 or past 450000 per CTA,
+                                    2 below 2^19 elements, else 4 (2 when the
                                     second buffer cannot be allocated);
                                 2 = pipelined in place: the next pivot's
                                     selection overlaps this pivot's update, no
@@ -170,9 +175,10 @@ typedef struct {
                                 one lp_solve call (or of lp_solve_async and the
                                 wait that completes it), 0 = none.  Past it the
                                 host raises an abort word in mapped host memory
-                                that every pivot kernel reads once per pass; the
-                                kernel stops within a pass and the solve ends in
-                                LP_TIMEOUT.  Ignored by batches, servers and
+                                that every pivot kernel reads once per pass (the
+                                panel kernel once per pivot, beside the device's
+                                own clock); the kernel stops within a pass and
+                                the solve ends in LP_TIMEOUT.  Ignored by batches, servers and
                                 lp_solve_noalloc.                               */
     int reinv_body;          /* FP32 mode, single LPs through lp_solve (not the
                                 servers, whose HBM budget has no room for the
@@ -251,9 +257,9 @@ typedef struct {
 
 /* Fill *opt with the defaults: FP64, reinv_k 50, max_iters 1e12, tolerances
  * by formula, bland_after 32, auto launch shape, spin timeout 4e9 cycles,
- * library stream, device 0, no trace, pipelined primal kernel, no wall-clock
- * limit, body refresh on, vectors left in place from 2^25 elements, no
- * spilling, three FP64 server lanes. */
+ * library stream, device 0, no trace, panel kernel, no wall-clock limit, body
+ * refresh on, columns that stay basic left out of the panels where m >= n / 4,
+ * no spilling, three FP64 server lanes. */
 void lp_options_default(lp_options *opt);
 
 /* Create a handle on opt->device (opt may be NULL for the defaults).
