@@ -583,6 +583,7 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     d.colx = h->dcolx;
     d.panel = h->dpanel;
     d.recs = h->dbar + kBarWords;
+    d.nonce = panel_nonce();
     d.abort = h->opt.time_limit_s > 0.0 ? h->dabort : nullptr;
     d.work = reinterpret_cast<unsigned long long *>(h->dbar + kBarWords + kPanelRecWords);
     CUDA_TRY(h, cudaMemsetAsync(d.work, 0, 2 * sizeof(unsigned long long), s));

@@ -81,7 +81,14 @@ struct LpDesc {
     // its records (2 exchanges x CTAs, a 128-byte line each; zeroed before a
     // launch)
     void *panel, *recs;
+    // and the tags of its values there: the load's number (panel_nonce) and the
+    // number of the last pivot, which goes on from launch to launch
+    unsigned nonce, epoch;
 };
+
+// A number no other load or batched launch of this process has: the panel
+// kernels' tags differ, whichever handle's memory they meet.
+unsigned panel_nonce();
 
 // Launch shape of the persistent pivot kernel for one LP.
 struct PivotShape {

@@ -369,7 +369,7 @@ enum : int { kJobEnd = 0, kJobCopy = 1, kJobPanel = 2, kJobInPlace = 3 };
 template <typename T, bool DUAL, int K, bool OV>
 __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g,
                                             long long spin_limit, long long budget, int drop,
-                                            unsigned nonce, long long limit_ns,
+                                            unsigned nonce, unsigned last_epoch, long long limit_ns,
                                             unsigned char *smem_raw) {
     typedef typename Vec<T>::type V;
     typedef typename DivisorOf<T>::type Divisor;
@@ -515,8 +515,8 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     int cur = 0, jobs = 0;
     // the slot of the pos-th pending pivot, oldest first
     auto slot = [&](int pos) { return !OV ? pos : pos < kold ? ho + pos : hn + pos - kold; };
-    unsigned epoch = 1;   // number of the pivot whose records are awaited
-    unsigned ecur = 1;    // number of the pivot being made
+    unsigned epoch = last_epoch + 1;  // number of the pivot whose records are awaited
+    unsigned ecur = epoch;            // number of the pivot being made
     int nodrop = 0;       // this panel gets every column
     int ab_next = 0;
     int last_p = d->last_p, last_q = d->last_q;
@@ -1565,6 +1565,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         d->deg = deg;
         d->last_p = last_p;
         d->last_q = last_q;
+        d->epoch = epoch;
         if (OV) {
             if (status != ST_TIMEOUT) d->T = Tab, d->T2 = bufs[cur ^ 1];
         } else if (d->work) {
@@ -1574,22 +1575,31 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     }
 }
 
+// The tags of one load's launches: its nonce, and pivot numbers that go on from
+// launch to launch.  Both are in the descriptor, not among the launch's
+// arguments, so a launch that was captured once and runs many times meets no
+// tag of an earlier run.
+__device__ __forceinline__ unsigned numbers_used(const LpDesc *d) {
+    return d->epoch < 0x80000000u ? d->epoch : 0u;
+}
+
 template <typename T, bool DUAL>
 __global__ void __launch_bounds__(kPanelThreads, 1)
     panel_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
-                 unsigned nonce, long long limit_ns) {
+                 long long limit_ns) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    panel_solve<T, DUAL, kPanelK, false>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, nonce,
-                                  limit_ns, smem_raw);
+    panel_solve<T, DUAL, kPanelK, false>(d, gridDim.x, blockIdx.x, spin_limit, budget, drop, d->nonce,
+                                         numbers_used(d), limit_ns, smem_raw);
 }
 
 template <bool DUAL>
 __global__ void __launch_bounds__(2 * kPanelThreads, 1)
     panel_overlap_kernel(LpDesc *__restrict__ d, long long spin_limit, long long budget, int drop,
-                         unsigned nonce, long long limit_ns) {
+                         long long limit_ns) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     panel_solve<double, DUAL, kPanelOverlapK, true>(d, gridDim.x, blockIdx.x, spin_limit, budget,
-                                                    drop, nonce, limit_ns, smem_raw);
+                                                    drop, d->nonce, numbers_used(d), limit_ns,
+                                                    smem_raw);
 }
 
 // Many LPs in one launch.  items[] lists (lp, rank) pairs, the ranks of one LP
@@ -1616,20 +1626,19 @@ __global__ void __launch_bounds__(kPanelThreads, 2)
         LpDesc *d = descs + w.x;
         if (d->sense)
             panel_solve<T, true, kPanelBatchK, false>(d, d->group, w.y, spin_limit, budget, drop, nonce,
-                                               0, smem_raw);
+                                               0, 0, smem_raw);
         else
             panel_solve<T, false, kPanelBatchK, false>(d, d->group, w.y, spin_limit, budget, drop, nonce,
-                                                0, smem_raw);
+                                                0, 0, smem_raw);
     }
 }
 
-// Tags of different launches differ, whichever handle's memory they meet.
-unsigned next_nonce() {
-    static std::atomic<unsigned> launches{0};
-    return ++launches;
-}
-
 }  // namespace
+
+unsigned panel_nonce() {
+    static std::atomic<unsigned> taken{0};
+    return ++taken;
+}
 
 PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop,
                               bool overlap) {
@@ -1666,9 +1675,8 @@ size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap) {
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s) {
     int drop = sh.drop;
-    unsigned nonce = next_nonce();
     long long limit_ns = sh.limit_ns;
-    void *args[] = {&d_desc, &spin_limit, &budget, &drop, &nonce, &limit_ns};
+    void *args[] = {&d_desc, &spin_limit, &budget, &drop, &limit_ns};
     const void *fn = sh.pipe == 5 ? (sh.dual ? (const void *)panel_overlap_kernel<true>
                                              : (const void *)panel_overlap_kernel<false>)
                      : prec == PREC_FP64 ? (sh.dual ? (const void *)panel_kernel<double, true>
@@ -1685,7 +1693,7 @@ cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long lo
 cudaError_t launch_panel_batch(int prec, LpDesc *descs, const int2 *items, int nitems,
                                unsigned *queue, int ctas, size_t smem, long long spin_limit,
                                long long budget, int drop, cudaStream_t s) {
-    unsigned nonce = next_nonce();
+    unsigned nonce = panel_nonce();
     void *args[] = {&descs, &items, &nitems, &queue, &spin_limit, &budget, &drop, &nonce};
     const void *fn = prec == PREC_FP64 ? (const void *)panel_batch_kernel<double>
                                        : (const void *)panel_batch_kernel<float>;

@@ -132,3 +132,46 @@ def test_overlapped_calls_that_end_around_a_panel(chunk, kind):
         assert np.array_equal(_bits(capi.lp_get_tableau(h, *A.shape)), _bits(o.T))
     finally:
         capi.lp_destroy(h)
+
+
+@pytest.mark.parametrize("sense", [MAX_LE, MIN_GE])
+@pytest.mark.parametrize("m,n", [(40, 30), (130, 90), (760, 690)])
+def test_captured_solve_runs_again(m, n, sense):
+    """A captured lp_solve_async, 7 pivots a run, run until the LP is solved,
+    then again after other LPs of the shape are loaded and begun (the largest
+    with overlapped panels): the values that carry tags are then those of earlier
+    runs of the same launch."""
+    import torch
+    stream = torch.cuda.Stream()
+    h = capi.lp_create(capi.lp_options_default(cuda_stream=stream, max_iters=7))
+    graph = None
+    try:
+        for seed in (1, 2, 1):
+            A, b, c = lpgen.paper_lp(m, n, seed=seed)
+            if sense == MIN_GE:
+                A, b, c = lpgen.dual_of(*lpgen.dense_lp(n, m, seed=seed))
+            capi.lp_load(h, A, b, c, sense)
+            torch.cuda.synchronize()
+            if graph is None:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream):
+                    capi.lp_solve_async(h)
+                first = 1
+            else:
+                capi.lp_solve(h)
+                first = 2
+            o = oracle.solve(A, b, c, sense=sense)
+            x, y = np.empty(A.shape[1]), np.empty(A.shape[0])
+            for run in range(first, o.iters // 7 + 3):
+                with torch.cuda.stream(stream):
+                    graph.replay()
+                obj, st, it = capi.lp_result(h, x, y)
+                assert it == min(7 * run, o.iters)
+                if st != capi.LP_ITER_LIMIT:
+                    break
+            assert st == o.status and it == o.iters and _bits([obj])[0] == _bits([o.obj])[0]
+            assert np.array_equal(_bits(x), _bits(o.x)) and np.array_equal(_bits(y), _bits(o.y))
+    finally:
+        torch.cuda.synchronize()
+        del graph
+        capi.lp_destroy(h)
