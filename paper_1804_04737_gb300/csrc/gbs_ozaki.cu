@@ -47,11 +47,11 @@
 // of a tableau row), and a copy-bound kernel writes the unit columns.  The
 // exponents and digits of the columns that remain, and so every bit written,
 // are those of the products over all columns.  At 8192 x 8192 with 50 to 334
-// structural basics the second product takes 0.88 ms and the unit columns
+// structural basics the second product takes 0.79 ms and the unit columns
 // 0.05, against 1.30 over all columns; with one MMA in six of the 334's it
-// takes as long, so its epilogue bounds it: by switching parts off, about 0.23
-// ms each are FP64 operations (two a value) and the sums' first steps, 0.14 the
-// reads of A.
+// takes as long, so its epilogue bounds it: by switching parts off, 0.23 ms are
+// FP64 operations (two a value), 0.14 the reads of A, 0.05 the digit groups'
+// sums.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -259,11 +259,10 @@ struct SrcRefreshB {  // row r: the groups' columns of [sg A_l | e_l], then sg b
     double sg;
     __device__ double at(int r, int e) const {
         const int l = R[r];
+        if (e < n) return sg * A[(long long)l * n + e];  // (the structurals' groups come first, all of them)
         if (e >= 4 * ng) return sg * b[l];
         const int g = grp[e >> 2], j = 4 * g + (e & 3);
-        if (g < 0) return 0.0;
-        if (j < n) return sg * A[(long long)l * n + j];
-        return (j - n == l) ? 1.0 : 0.0;
+        return g >= 0 && j - n == l ? 1.0 : 0.0;
     }
 };
 
@@ -336,17 +335,28 @@ __global__ void oz_rowexp_kernel(Src src, int M, int K, const int *shift, int *r
     if (lane == 0) rowexp[w] = mx;
 }
 
-// Largest shifted exponent of each column j < N of B over k < K.
+// Largest shifted exponent of each column j < N of B over k < K: 32 columns per
+// block of 256, eight rows at once (one thread per column, K rows in turn, left
+// most of the chip idle).
 template <class Src>
-__global__ void oz_colexp_kernel(Src src, int K, int N, const int *shift, int *colexp) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
+__global__ void __launch_bounds__(256) oz_colexp_kernel(Src src, int K, int N, const int *shift,
+                                                        int *colexp) {
+    __shared__ int red[8][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, j = blockIdx.x * 32 + tx;
     int mx = kNoExp;
-    for (int k = 0; k < K; ++k) {
-        const int ex = exp_of(src.at(k, j));
-        if (ex) mx = max(mx, ex - shift[k]);
+    if (j < N) {
+#pragma unroll 4
+        for (int k = ty; k < K; k += 8) {
+            const int ex = exp_of(src.at(k, j));
+            if (ex) mx = max(mx, ex - shift[k]);
+        }
     }
-    colexp[j] = mx;
+    red[ty][tx] = mx;
+    __syncthreads();
+    if (ty == 0 && j < N) {
+        for (int r = 1; r < 8; ++r) mx = max(mx, red[r][tx]);
+        colexp[j] = mx;
+    }
 }
 
 // A digit planes: out[p][i][k] (Mp x Kp per plane), zero in the padding.
@@ -742,7 +752,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             const double *arow = p.Aorig;
             double av[8];
             // (rows of A on 32 bytes, as the groups are: one read per group
-            // instead of four, and the rounding by integers: 1.02 -> 0.88 ms)
+            // instead of four, and the rounding by integers: 1.02 -> 0.88 ms; this
+            // mode's own instance 0.79)
             const bool quads = ((p.n & 3) | (int)((unsigned long long)p.Aorig & 31)) == 0;
             auto orig = [&](double (&x)[8], int ja, int jb) {
                 if (quads) {
@@ -982,7 +993,7 @@ cudaError_t oz_product(SA srcA, SB srcB, int M, int N, int K, OzParams p, OzWork
         else oz_kexpB_kernel<SB, false><<<(K + 7) / 8, 256, 0, s>>>(srcB, K, Nb, kA, shift);
     }
     oz_rowexp_kernel<SA><<<(M + 7) / 8, 256, 0, s>>>(srcA, M, K, shift, w.rowexp);
-    oz_colexp_kernel<SB><<<(N + 255) / 256, 256, 0, s>>>(srcB, K, N, shift, w.colexp);
+    oz_colexp_kernel<SB><<<(N + 31) / 32, 256, 0, s>>>(srcB, K, N, shift, w.colexp);
     {
         const long long total = (long long)Mp * Kp;
         const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * sms * 8);
