@@ -78,6 +78,7 @@
 #include <atomic>
 #include <type_traits>
 
+#include "gbs_colbits.h"
 #include "gbs_device.cuh"
 #include "gbs_internal.h"
 
@@ -328,7 +329,7 @@ __host__ __device__ inline PanelLayout panel_layout(int m, int N, int G, int esz
     L.stay = take((size_t)L.nwords * sizeof(unsigned));
     L.prev = take(ov ? (size_t)L.nwords * sizeof(unsigned) : 0);
     L.out = take(ov ? (size_t)L.nwords * sizeof(unsigned) : 0);
-    L.list = take((size_t)L.nvec * sizeof(int));
+    L.list = take((size_t)L.nwords * (32 / vw) * sizeof(int));
     L.total = at;
     return L;
 }
@@ -478,7 +479,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         cta_sync();
         for (int w = tid; w < nwords; w += B) {
             // (columns past the last one never need an update)
-            if (w == nwords - 1 && (N & 31)) bb[w] |= ~0u << (N & 31);
+            bb[w] |= past_end(w, N);
             stay[w] = bb[w];
             if (OV) prev[w] = ~0u;  // (the copy makes the buffers equal)
         }
@@ -565,7 +566,6 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         const int bw = bt >> 5;
         // the vectors to update, in order
         int nact;
-        constexpr unsigned full = (1u << VW) - 1u;
         if (bt == 0) s_task = 0;
         if (all) {
             for (int v = bt; v < nvec; v += B) list[v] = v;
@@ -577,7 +577,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             int cnt = 0;
             for (int w = w0; w < w1; ++w) {
                 const unsigned s = left_out[w];
-                for (int u = 0; u < 32 / VW; ++u) cnt += (s >> (u * VW) & full) != full;
+                for (int u = 0; u < 32 / VW; ++u) cnt += vector_kept(s, u, VW);
             }
             int pre = cnt;
 #pragma unroll
@@ -597,7 +597,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             for (int w = w0; w < w1; ++w) {
                 const unsigned s = left_out[w];
                 for (int u = 0; u < 32 / VW; ++u)
-                    if ((s >> (u * VW) & full) != full) list[at++] = w * (32 / VW) + u;
+                    if (vector_kept(s, u, VW)) list[at++] = w * (32 / VW) + u;
             }
             sync();
         }
@@ -675,7 +675,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 V *const to = reinterpret_cast<V *>(dst + (long long)(i0 + r) * P);
                 for (int v = bt; v < nvec; v += B) {
                     const int j = v * VW;
-                    if ((left_out[j >> 5] >> (j & 31) & full) != full) continue;
+                    if (vector_kept(left_out[j >> 5], (j & 31) / VW, VW)) continue;
                     V x = ldv(from + v);
                     for (int t = 0; t < kk; ++t) {
                         const V pt = ldv(reinterpret_cast<const V *>(PR + (h + t) * P) + v);
@@ -1294,9 +1294,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 if (jobs > 1) cur ^= 1, Tab = bufs[cur];
                 const bool all = !drop || nodrop;
                 for (int w = tid; w < nwords; w += B) {
-                    const unsigned s = stay[w];
-                    out[w] = prev[w] & s;
-                    prev[w] = all ? 0u : s;
+                    out[w] = left_out_of_panel(prev[w], stay[w], all, past_end(w, N));
                     stay[w] = bb[w];
                 }
                 for (int r = tid; r < R; r += B)  // (the other half's slots are used again)
