@@ -52,9 +52,13 @@
 // 32 bytes between records took 10 to 30% longer per pivot, and a counter
 // released after the records 3960 clocks).  Polling starts once the CTA's own
 // record is out: polls from the start of the pivot doubled the exchange.
-// What else crosses CTAs (single entries of pending rows and columns, a
-// record's further values) carries its pivot's tag beside it, so no fence
-// orders it: fences took 450 clocks alone and 3000 under the polls.
+// What else crosses CTAs for a pivot (single entries of pending rows and
+// columns, a record's further values) carries its pivot's tag beside it, so no
+// fence orders it: fences took 450 clocks alone and 3000 under the polls.  What
+// a panel reads (the pending rows, plain) and writes (the tableau) has no tags
+// and is ordered once per panel: the lane that publishes the record which
+// announces it fences first, after the barrier that follows the writes, and the
+// lanes that poll that record fence before the barrier that precedes the reads.
 //
 // Columns that stay basic through a panel are exact unit vectors: their
 // entries in its pivot rows are zeros, and an fma with a zero product leaves a
@@ -686,8 +690,10 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 }
             }
         }
-        __threadfence();  // other CTAs read these rows after this CTA's next record
+        // other CTAs read these rows after this CTA's next record: whichever
+        // thread publishes it, its fence follows every thread's writes
         sync();
+        __threadfence();
     };
     // The pending pivots of a full or last panel, in place (not OV).
     auto apply_panel = [&](int kk) {
@@ -712,8 +718,8 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 const long long cnt = (long long)R * pv;
 #pragma unroll 4
                 for (long long e = bt; e < cnt; e += B) dst[e] = ldv(src + e);
-                __threadfence();
                 sync();
+                __threadfence();
             } else {
                 T *const src = bufs[s_job[3]];
                 panel_job(src, kind == kJobPanel ? bufs[s_job[3] ^ 1] : src, s_job[1], s_job[2],
@@ -738,9 +744,11 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     };
     // OV: wait for the jobs posted; they have no waits of their own.
     auto wait_jobs = [&]() {
-        if (lane == 0)
+        if (lane == 0) {
             while (*(volatile int *)&s_done != jobs) {
             }
+            __threadfence_block();
+        }
         __syncwarp();
     };
     // Every CTA of the group; false when a wait ran out.
@@ -851,10 +859,11 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     auto open_gate = [&](int id) {
         if (G > 1 && !poll_warp) group_arrive(id, id == 3 ? gate3 : gate4);
     };
-    // The records of this lane in a poll warp, of pivot `epoch`.  (One failure
+    // The records of this lane in a poll warp, of pivot `epoch`; acquire: they
+    // announce untagged data.  (One failure
     // flag per exchange: one exchange's flag is read by every thread before a
     // warp can be polling in the same exchange again.)
-    auto poll = [&](int which, ulonglong2 (&v)[kPollRecs]) {
+    auto poll = [&](int which, ulonglong2 (&v)[kPollRecs], bool acquire) {
         const int id = (which != 0) == DUAL ? 3 : 4;
         group_sync(id, id == 3 ? gate3 : gate4);
         const int e0 = (wid - kPollFirst) * 32 + lane;
@@ -874,6 +883,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 break;
             }
         }
+        if (acquire) __threadfence();
     };
 
     // Exchange 1: the smallest record 1 (Dantzig: by value, ties smallest
@@ -904,7 +914,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         }
         if (poll_warp) {
             ulonglong2 v[kPollRecs];
-            poll(0, v);
+            poll(0, v, k == K);  // (a full panel is applied next)
             const int e0 = (wid - kPollFirst) * 32 + lane;
             unsigned long long vk = ~0ull, x = 0;
             int key = 0x7fffffff, idx = -1, e = e0, flag = 0;
@@ -965,7 +975,9 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         unsigned sk[kPollRecs];
         const int e0 = (wid - kPollFirst) * 32 + lane;
         if (poll_warp) {
-            poll(1, v);
+            // (in turn: row p is read next, perhaps as the panel just left it; the
+            // dual rule has read it already, behind a barrier)
+            poll(1, v, !OV && !DUAL && k == 0);
             unsigned b1 = kNone, b2 = kNone, flag = 0;
             int at = 0;
 #pragma unroll
@@ -1223,8 +1235,9 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             }
         }
     };
-    // Records 1 of the dual rule (row warps): the leaving row.
-    auto publish_leaving = [&](bool bland, int flag) {
+    // Records 1 of the dual rule (row warps): the leaving row.  release: it
+    // announces untagged data.
+    auto publish_leaving = [&](bool bland, int flag, bool release) {
         unsigned long long vk = ~0ull;
         int key = 0x7fffffff, loc = -1;
         for (int r = rt; r < R; r += B) {
@@ -1235,6 +1248,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             if (v < vk || (v == vk && ky < key)) vk = v, key = ky, loc = r;
         }
         local_min(2, nw - 1 - wid, rw, vk, key, loc, flag, [&](int l, unsigned fl) {
+            if (release && G > 1) __threadfence();
             if (l < 0) {
                 publish(0, 0ull, -1, fl);
             } else {
@@ -1246,8 +1260,9 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         });
     };
     // Records 1 of the primal rule (column warps): the entering column.
-    auto publish_entering = [&](unsigned long long vk, int loc, int flag) {
+    auto publish_entering = [&](unsigned long long vk, int loc, int flag, bool release) {
         local_min(1, wid, cw, vk, loc < 0 ? 0x7fffffff : loc, loc, flag, [&](int c, unsigned fl) {
+            if (release && G > 1) __threadfence();
             publish(0, c < 0 ? 0ull : to_bits(zs[c]), c < 0 ? -1 : c0 + c, fl);
         });
     };
@@ -1264,11 +1279,11 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             const unsigned long long v = bland ? zero_k : zk;
             if (v < vk) vk = v, loc = c;
         }
-        publish_entering(vk, loc, 0);
+        publish_entering(vk, loc, 0, false);
         open_gate(3);
     }
     if (DUAL && row_warp) {
-        publish_leaving(deg >= bland_after, 0);
+        publish_leaving(deg >= bland_after, 0, false);
         open_gate(4);
     }
 
@@ -1492,16 +1507,12 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 }
             }
             __syncwarp();
-            // a full panel is applied after the next records: the rows it
-            // reads, and what the panel before it wrote, must have arrived
-            // before this CTA's record says so
-            if (kc + 1 == K) {
-                if (OV) wait_jobs();
-                if (G > 1) __threadfence();
-            }
+            // a full panel is applied after the next records: this CTA's
+            // announces the rows it reads, and what the panel before it wrote
             if (!DUAL) {
+                if (OV && kc + 1 == K) wait_jobs();
                 k = kc + 1;
-                publish_entering(vk, loc, flag);
+                publish_entering(vk, loc, flag, kc + 1 == K);
                 open_gate(3);
             }
         }
@@ -1520,7 +1531,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 update_rhs(hn + kc, p, q, lane_value(f, kRhs1),
                            Divisor(lane_value(f, kDen2), lane_value(f, kRcp2)));
                 __syncwarp();
-                publish_leaving(nbland, bad);
+                publish_leaving(nbland, bad, kc + 1 == K);
                 open_gate(4);
             }
         } else if (row_warp) {
