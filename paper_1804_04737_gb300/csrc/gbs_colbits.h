@@ -36,4 +36,15 @@ GBS_HD unsigned left_out_of_panel(unsigned &prev, unsigned stay, bool all, unsig
     return out;
 }
 
+// A pivot: column `leaving` is basic no more (nor has it stayed so), column
+// `entering` is.  `leaving` may be any bits once the wait for it ran out (the
+// solve then ends at its next exchange): outside the N columns it marks nothing.
+GBS_HD void change_basis(unsigned *basic, unsigned *stay, int leaving, int entering, int N) {
+    if (leaving >= 0 && leaving < N) {
+        basic[leaving >> 5] &= ~(1u << (leaving & 31));
+        stay[leaving >> 5] &= ~(1u << (leaving & 31));
+    }
+    basic[entering >> 5] |= 1u << (entering & 31);
+}
+
 }  // namespace gbs

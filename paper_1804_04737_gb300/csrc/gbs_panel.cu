@@ -1453,9 +1453,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             if (DUAL)
                 var = (int)__shfl_sync(kAll, fetch(nullptr, 0, nullptr, e1.cta, -1, 0), kVar1);
             if (lane == 0) {
-                bb[var >> 5] &= ~(1u << (var & 31));
-                stay[var >> 5] &= ~(1u << (var & 31));
-                bb[q >> 5] |= 1u << (q & 31);
+                change_basis(bb, stay, var, q, N);
                 if (g == 0 && iters <= trace_cap) {
                     d->trace[2 * iters - 2] = p;
                     d->trace[2 * iters - 1] = q;

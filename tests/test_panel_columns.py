@@ -56,6 +56,38 @@ int main() {
 }
 """
 
+BASIS = r"""
+#include <climits>
+#include <cstdio>
+#include <cstring>
+#include <initializer_list>
+#include "gbs_colbits.h"
+
+int main() {
+    int bad = 0;
+    for (int N : {1, 31, 32, 33, 70}) {
+        const int nwords = (N + 31) / 32;
+        for (int leaving : {0, N / 2, N - 1, N, N + 1, 32 * nwords, 1 << 20, INT_MAX, -1, -33, INT_MIN}) {
+            unsigned mem[16], want[16];  // guards, basic, guards, stay, guards
+            for (unsigned &w : mem) w = 0xffffffffu;
+            std::memcpy(want, mem, sizeof mem);
+            unsigned *basic = mem + 2, *stay = mem + 9;
+            const int entering = N / 3;
+            basic[entering / 32] &= ~(1u << entering % 32);
+            want[2 + entering / 32] |= 1u << entering % 32;
+            if (leaving >= 0 && leaving < N) {
+                if (leaving != entering) want[2 + leaving / 32] &= ~(1u << leaving % 32);
+                want[9 + leaving / 32] &= ~(1u << leaving % 32);
+            }
+            gbs::change_basis(basic, stay, leaving, entering, N);
+            bad += std::memcmp(mem, want, sizeof mem) != 0;
+        }
+    }
+    std::printf("%d\n", bad);
+    return bad != 0;
+}
+"""
+
 
 def _run(tmp_path, source):
     src, exe = tmp_path / "cols.cpp", tmp_path / "cols"
@@ -67,4 +99,9 @@ def _run(tmp_path, source):
 
 def test_panels_list_only_their_own_vectors(tmp_path):
     r = _run(tmp_path, PANELS)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_leaving_column_out_of_range_marks_nothing(tmp_path):
+    r = _run(tmp_path, BASIS)
     assert r.returncode == 0, r.stdout + r.stderr
