@@ -387,7 +387,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     __shared__ __align__(16) T s_at[nw][KS];  // a warp's pending entries at one row or column
     __shared__ int s_flag, s_fail[2], s_nflag, s_task, s_scan[nw];
     __shared__ int s_prow[NS];  // pivot rows of the pending pivots
-    __shared__ int s_job[5], s_done;  // OV: the panel to apply, panels applied
+    __shared__ int s_job[5];    // OV: the panel to apply
     __shared__ ulonglong2 s_rec[2];
     __shared__ unsigned long long s_aux[2][2][4];
 
@@ -473,7 +473,6 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         if (tid == 0) {
             s_fail[0] = s_fail[1] = 0;
             s_nflag = 0;
-            s_done = 0;
         }
         cta_sync();
         for (int i = tid; i < m; i += B) {
@@ -708,7 +707,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     if (OV && tid >= B) {
         const int bt = tid - B;
         auto sync = [&]() { group_sync(6, nw); };
-        for (int done = 1;; ++done) {
+        for (;;) {
             group_sync(7, 2 * nw);
             const int kind = s_job[0];
             if (kind == kJobEnd) break;
@@ -725,7 +724,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
                 panel_job(src, kind == kJobPanel ? bufs[s_job[3] ^ 1] : src, s_job[1], s_job[2],
                           s_job[4] != 0, out, bt, sync);
             }
-            if (bt == 0) *(volatile int *)&s_done = done;
+            group_arrive(8, 2 * nw);
         }
         if (g == 0 && bt == 0 && d->work) {
             d->work[0] += upd;
@@ -742,14 +741,14 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         group_arrive(7, 2 * nw);
         ++jobs;
     };
-    // OV: wait for the jobs posted; they have no waits of their own.
-    auto wait_jobs = [&]() {
-        if (lane == 0) {
-            while (*(volatile int *)&s_done != jobs) {
-            }
-            __threadfence_block();
-        }
+    // OV: wait until the job posted last is done (once per job, every selection
+    // warp; one that does not read what the job wrote only arrives).  A barrier:
+    // polling a flag in shared memory would be a wait without a limit, and no
+    // job may be posted while one is under way.
+    auto wait_job = [&](bool here) {
         __syncwarp();
+        if (here) group_sync(8, 2 * nw);
+        else group_arrive(8, 2 * nw);
     };
     // Every CTA of the group; false when a wait ran out.
     auto group_barrier = [&]() {
@@ -1508,7 +1507,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             // a full panel is applied after the next records: this CTA's
             // announces the rows it reads, and what the panel before it wrote
             if (!DUAL) {
-                if (OV && kc + 1 == K) wait_jobs();
+                if (OV && kc + 1 == K) wait_job(true);
                 k = kc + 1;
                 publish_entering(vk, loc, flag, kc + 1 == K);
                 open_gate(3);
@@ -1521,7 +1520,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             if (row_warp) bad = form_col(q, e1.cta, e2.cta, 0, &f);
             // (as above; the row warps publish, the column warps wrote the rows)
             if (kc + 1 == K) {
-                if (OV) wait_jobs();
+                if (OV) wait_job(true);
                 cta_sync();
             }
             k = kc + 1;
@@ -1537,13 +1536,14 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             update_rhs(hn + kc, p, q, lane_value(f, kNum2),
                        Divisor(lane_value(f, kDen2), lane_value(f, kRcp2)));
         }
+        if (OV && !DUAL && !col_warp && kc + 1 == K) wait_job(false);
         k = kc + 1;
         if (tid == 0) s_prow[hn + kc] = p;
     }
 
     // --------------------------------------------------------------- end --
     if constexpr (OV) {
-        wait_jobs();
+        if (k < K) wait_job(true);  // (at the last pivot of a panel it was waited for)
         // (every CTA takes this branch: the records decide, and they agree)
         if (status != ST_TIMEOUT && !group_barrier()) status = ST_TIMEOUT;
         if (status != ST_TIMEOUT) {
@@ -1551,7 +1551,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             if (k > 0) {
                 for (int w = tid; w < nwords; w += B) out[w] = stay[w];
                 post(kJobInPlace, hn, k, !drop || nodrop);
-                wait_jobs();
+                wait_job(true);
             }
         }
         post(kJobEnd, 0, 0, false);
