@@ -296,8 +296,10 @@ __global__ void oz_kexpA_kernel(Src src, int M, int K, int *kA) {
 }
 
 // eB_k: largest exponent of row k of B (K x N), one block of 256 per k
-// (kWide) or one warp; then shift_k.  Long rows get a block: with one warp, 334
-// rows of 16385 took 136 us, most of the chip idle.
+// (kWide) or one warp; then shift_k.  A block where one warp per row would leave
+// SMs idle and the row has a column for each thread.  Measured, us, warp / block:
+// 334 rows of 256 columns 3.0 / 3.1, 500 4.0 / 3.7, 4000 9.3 / 6.7; 100 of 16385
+// 24 / 13; 2000 rows of 256 3.9 / 4.9, 1000 7.9 / 8.1, 4000 13.8 / 14.1.
 template <class Src, bool kWide>
 __global__ void __launch_bounds__(256) oz_kexpB_kernel(Src src, int K, int N, const int *kA, int *shift) {
     __shared__ int red[8];
@@ -305,10 +307,15 @@ __global__ void __launch_bounds__(256) oz_kexpB_kernel(Src src, int K, int N, co
     const int k = kWide ? (int)blockIdx.x : (int)(blockIdx.x * 8 + warp);
     int mx = kNoExp;
     if (k < K) {
-#pragma unroll 4
-        for (int j = kWide ? threadIdx.x : lane; j < N; j += kWide ? 256 : 32) {
+        auto take = [&](int j) {
             const int ex = exp_of(src.at(k, j));
             if (ex) mx = max(mx, ex);
+        };
+        if (kWide) {
+#pragma unroll 4
+            for (int j = threadIdx.x; j < N; j += 256) take(j);
+        } else {  // (unrolled by hand it took half as long again from 500 columns on)
+            for (int j = lane; j < N; j += 32) take(j);
         }
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
@@ -989,7 +996,7 @@ cudaError_t oz_product(SA srcA, SB srcB, int M, int N, int K, OzParams p, OzWork
         if ((e = cudaMemsetAsync(kA, 0, sizeof(int) * (size_t)K, s)) != cudaSuccess) return e;
         oz_kexpA_kernel<SA><<<dim3((K + 31) / 32, (M + 63) / 64), 256, 0, s>>>(srcA, M, K, kA);
         const int Nb = std::max(N, Nexp);
-        if (Nb >= 2048) oz_kexpB_kernel<SB, true><<<K, 256, 0, s>>>(srcB, K, Nb, kA, shift);
+        if (Nb > 256 && K < 8 * sms) oz_kexpB_kernel<SB, true><<<K, 256, 0, s>>>(srcB, K, Nb, kA, shift);
         else oz_kexpB_kernel<SB, false><<<(K + 7) / 8, 256, 0, s>>>(srcB, K, Nb, kA, shift);
     }
     oz_rowexp_kernel<SA><<<(M + 7) / 8, 256, 0, s>>>(srcA, M, K, shift, w.rowexp);
