@@ -516,6 +516,22 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// Lane l of each half-warp holds x[0..15] of row l; afterwards it holds column l
+// of rows 0..15.  (Four exchanges, one per bit: element and lane change places.)
+__device__ __forceinline__ void transpose16(double (&x)[16], int lane) {
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+        const bool up = lane & d;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (i & d) continue;
+            const double y = __shfl_xor_sync(0xffffffffu, up ? x[i] : x[i | d], d);
+            if (up) x[i] = y;
+            else x[i | d] = y;
+        }
+    }
+}
+
 // Four doubles at p + j (32-byte aligned), zeros where j is outside [0, n).
 __device__ __forceinline__ void ldg4(const double *p, int j, int n, double *x) {
     x[0] = x[1] = x[2] = x[3] = 0.0;
@@ -831,23 +847,34 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tmem_empty);
-                    // Each thread writes its own row's results (the row its
-                    // tensor-memory lane holds): one contiguous row segment per
-                    // thread, read (C, or the original row of A) and written with
-                    // independent accesses, no shared-memory transposition.
+                    // Mode 0: each lane holds 16 columns of its own row; an exchange
+                    // in the warp gives it one column of 16 rows, so that a store
+                    // writes 128 bytes of each of two rows.  (Stores of each thread's
+                    // own row, 8 bytes in 32 rows at a time, bounded the tile where
+                    // the MMAs are few, more so with 16 columns a thread than with 8:
+                    // 7858 x 16385 x 100 1.56 ms, 1.44 with 8 at a time, 0.94 so; x 40
+                    // 1.48, 0.85 so; x 334 1.76, 1.59 so.)
                     if constexpr (MODE == 0) {
-                        if (r < p.M) {
-                            double *crow = p.C + (long long)r * p.ldc + j0;
+                        double x[16];
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                const int Fc = s_colexp[cb + j];
-                                double v = 0.0;
-                                // scale 2^(Er - 1022 + Fc - 1022 - 14)
-                                if (Er != kNoExp && Fc != kNoExp) v = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
-                                if (j0 + j < p.N) crow[j] = c == 0 ? v : crow[j] + v;
-                            }
+                        for (int j = 0; j < 16; ++j) {
+                            const int Fc = s_colexp[cb + j];
+                            x[j] = 0.0;
+                            // scale 2^(Er - 1022 + Fc - 1022 - 14)
+                            if (Er != kNoExp && Fc != kNoExp) x[j] = scaled_sum(hi[j], lo[j], Er + Fc - 2058);
+                        }
+                        transpose16(x, lane);
+                        const int col = j0 + (lane & 15), r0 = m0 + lg * 32 + (lane & 16);
+                        if (col < p.N) {
+                            double *at = p.C + (long long)r0 * p.ldc + col;
+#pragma unroll
+                            for (int j = 0; j < 16; ++j, at += p.ldc)
+                                if (r0 + j < p.M) *at = c == 0 ? x[j] : *at + x[j];
                         }
                     } else if (r < p.M) {
+                        // Each thread writes its own row's results: one contiguous
+                        // row segment, the original row of A read and the tableau
+                        // written with independent 16-byte accesses.
                         const long long sgbit = p.sg < 0.0 ? (long long)kSign : 0ll;
                         float *trow = p.T32 + (long long)ti * p.P;
                         double aw[8];

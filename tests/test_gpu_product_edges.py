@@ -3,7 +3,8 @@
 Integer matrices whose products are exact in FP64 (entries below 2^10), so the
 result is numpy's bit for bit, on either side of the sizes where the row
 exponents of B go from a warp to a block per row (256 columns; a row for each
-eight SMs' warps).
+eight SMs' warps), and where its results, exchanged between the lanes of a warp
+so that 16 columns of a row are written together, end inside such a piece.
 """
 import ctypes
 
@@ -37,3 +38,27 @@ def test_row_exponents(N, K):
     C = torch.empty((40, N), dtype=torch.float64, device="cuda")
     capi.lp_dgemm_emulated(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C)
     assert np.array_equal(C.cpu().numpy(), A @ B)
+
+
+@pytest.mark.parametrize("K", [1, 64, 65, 449])
+@pytest.mark.parametrize("M", [1, 15, 16, 17, 31, 33, 127, 129])
+def test_ragged_results_and_pitches(M, K):
+    """Results of every width around a piece, a warp's columns and a tile, in a
+    matrix with a longer pitch that starts 8 bytes off a 16-byte boundary: the
+    entries around them keep their bits."""
+    lib = capi.load_library()
+    rng = np.random.default_rng(M + K)
+    A = _ints(rng, M, K)
+    tA = torch.from_numpy(A).cuda()
+    for N in (1, 15, 16, 17, 47, 63, 64, 65, 130):
+        B = _ints(rng, K, N)
+        tB = torch.from_numpy(B).cuda()
+        for pitch in (N, N + 3):
+            mem = torch.full((M * pitch + 10,), np.nan, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            assert lib.lp_dgemm_emulated(M, N, K, tA.data_ptr(), K, tB.data_ptr(), N,
+                                         mem.data_ptr() + 40, pitch, None) == 0
+            got = mem.cpu().numpy()
+            want = np.full(M * pitch + 10, np.nan)
+            np.lib.stride_tricks.as_strided(want[5:], (M, N), (8 * pitch, 8))[:] = A @ B
+            assert np.array_equal(got, want, equal_nan=True)
