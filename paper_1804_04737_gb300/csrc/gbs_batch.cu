@@ -299,8 +299,6 @@ lp_err solve_batch_fp32(const BatchFp32 &f, lp_status *fin, double *kernel_ms) {
             budget = std::min(budget, remaining[k]);
             for (int r = 0; r < f.G[k]; ++r) f.h_items[nitems++] = make_int2(k, r);
             f.h_desc[k].sense = rule[k];
-            // (the dual rule's negative pivots leave -0 in basic columns)
-            if (rule[k]) f.h_desc[k].negz = 1;
             before[k] = f.h_desc[k].iters;
         }
         if (nitems == 0) break;

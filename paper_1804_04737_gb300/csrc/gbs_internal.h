@@ -75,9 +75,11 @@ struct LpDesc {
     unsigned long long *work;
     // nonzero when a constraint row may hold a -0 (from the data, Phase I,
     // FP32 mode, or a -0 an update produced): no vector is left in place; bit 1:
-    // the basic columns are known to be exact unit vectors with +0 elsewhere
+    // a refresh has made the basic columns exact unit vectors with +0 elsewhere
+    // since the last launch
     int negz;
-    // panel kernel: its pending columns and rows (panel_workspace bytes), and
+    // panel kernel: its pending columns and rows and, from launch to launch, its
+    // marks on rows (panel_workspace bytes), and
     // its records (2 exchanges x CTAs, a 128-byte line each; zeroed before a
     // launch)
     void *panel, *recs;

@@ -65,10 +65,12 @@
 // finite nonzero entry and +0 as they are.  The panel leaves such columns out
 // (lp_options.zero_skip).  Exceptions are tracked: a pivot row divided by a
 // negative pivot (dual rule) holds -0 in them, so its row is marked and marked
-// rows get every column; a launch that finds the tableau already pivoted by
-// the dual rule or refreshed scans its rows for such entries first; and a
-// panel with a non-finite pivot column, or with a nonzero pivot-row entry in a
-// column thought to stay, gets every column in every row.
+// rows get every column; the marks are kept in memory from launch to launch, up
+// to a refresh, which writes exact unit vectors (finding such rows by a scan
+// took longer than a launch of a few pivots: 512 x 4096, dual, one pivot a call,
+// 1.5 times the call); and a panel with a non-finite pivot column, or with a
+// nonzero pivot-row entry in a column thought to stay, gets every column in
+// every row.
 //
 // Waits are bounded: a poll that does not succeed within the spin limit sets
 // the error flag and the kernel returns with status TIMEOUT.
@@ -406,6 +408,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     ulonglong2 *const PT = CT + (G > 1 ? NS * Mp : 0);
     ulonglong2 *const AX = PT + (G > 1 ? NS * Np : 0);
     T *const PR = reinterpret_cast<T *>(AX + (G > 1 ? 16 * G : 0));
+    unsigned char *const marks = reinterpret_cast<unsigned char *>(PR + NS * P);  // rowz, between launches
     ulonglong2 *const recs = reinterpret_cast<ulonglong2 *>(d->recs);
     int *const err = d->err;
 
@@ -449,7 +452,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         iters > 0x3fffffffffffffffll - budget ? 0x3fffffffffffffffll : iters + budget;
     int deg = d->deg;
     int status = ST_RUNNING;
-    const bool scan = drop && iters > 0 && (DUAL || d->negz) && !(d->negz & 2);
+    const bool marked = iters > 0 && !(d->negz & 2);
     const int *const abort_word = d->abort;
     const unsigned long long t_start = limit_ns > 0 ? global_ns() : 0ull;
     const long long trace_cap = d->trace_cap;
@@ -461,7 +464,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         for (int r = tid; r < R; r += B) {
             rh[r] = lds(Tab + (long long)(i0 + r) * P + (N - 1));
             bas[r] = __ldcg(d->basis + i0 + r);
-            rowz[r] = 0;
+            rowz[r] = marked ? __ldcg(marks + i0 + r) : 0;
             lastp[r] = -1;
         }
         for (int w = tid; w < nwords; w += B) bb[w] = 0;
@@ -486,30 +489,8 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             stay[w] = bb[w];
             if (OV) prev[w] = ~0u;  // (the copy makes the buffers equal)
         }
-        if (scan) {
-            // rows whose entries in basic columns are not all +0 (but the
-            // unit entry): -0 from the dual rule or a refresh
-            cta_sync();
-            for (int r = wid; r < R; r += nw) {
-                const T *row = Tab + (long long)(i0 + r) * P;
-                int bad = 0;
-                for (int j0 = 0; j0 < N; j0 += 256) {
-                    T x[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) x[u] = lds(row + min(j0 + 32 * u + lane, N - 1));
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int j = j0 + 32 * u + lane;
-                        bad |= j < N && (bb[(j0 >> 5) + u] >> lane & 1u) && j != bas[r] &&
-                               to_bits(x[u]) != 0ull;
-                    }
-                }
-                if (__any_sync(kAll, bad) && lane == 0) {
-                    rowz[r] = 1;
-                    s_nflag = 1;
-                }
-            }
-        }
+        for (int r = tid; r < R; r += B)
+            if (rowz[r]) s_nflag = 1;
         cta_sync();
     }
 
@@ -1563,7 +1544,7 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
     {
         T *z = Tab + (long long)m * P;
         for (int c = tid; c < W; c += B) z[c0 + c] = zs[c];
-        for (int r = tid; r < R; r += B) d->basis[i0 + r] = bas[r];
+        for (int r = tid; r < R; r += B) d->basis[i0 + r] = bas[r], marks[i0 + r] = rowz[r];
     }
     if (g == 0 && tid == 0) {
         d->status = (*(volatile int *)err) ? ST_TIMEOUT : status;
@@ -1672,7 +1653,7 @@ size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K) 
     const size_t esz = prec == PREC_FP64 ? 8 : 4;
     const size_t tagged =
         G > 1 ? (size_t)K * (size_t)(tag_pitch(m) + tag_pitch(N)) * 16 + 256 * (size_t)G : 0;
-    return tagged + (size_t)K * (size_t)P * esz;
+    return tagged + (size_t)K * (size_t)P * esz + (size_t)m;
 }
 
 size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap) {
