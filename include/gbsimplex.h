@@ -139,13 +139,17 @@ typedef struct {
                                     demand and applied to the tableau up to 16
                                     at a time in place or, in FP64 from 2^20
                                     tableau elements ((m+1) x row pitch) up to
-                                    450000 per CTA, up to 8 at a time into a
+                                    450000 per CTA with at least 64 rows and
+                                    columns and not few pivots to make
+                                    (max_iters), up to 8 at a time into a
                                     second buffer (in place where it cannot be
                                     allocated) while the next are selected;
                                     where the panel kernel cannot take the LP
                                     (its workspace or its shared memory does
                                     not fit), and with n > 4 m from 2^20
-                                    elements on in FP32 or past 450000 per CTA,
+                                    elements on when not into a second buffer,
+                                    or with fewer than 16 rows, or where rows
+                                    are long for the rows per CTA,
                                     2 below 2^19 elements, else 4 (2 when the
                                     second buffer cannot be allocated);
                                 2 = pipelined in place: the next pivot's

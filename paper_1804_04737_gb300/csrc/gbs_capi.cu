@@ -56,6 +56,37 @@ constexpr long long kSkipElems = 1ll << 25;
 // the selection they hide.
 constexpr long long kOverlapElems = 1ll << 20;
 constexpr long long kOverlapPerCta = 450000;
+// Few pivots run their panels in turn all the same: the overlapped kernel would
+// copy the whole tableau first, and fill no panel to hide.  That is a launch of
+// fewer pivots than this (twelve calls of so many, us in turn / overlapped:
+// 2048^2 (8.5 M elements) 1 pivot 1027 / 1662, 8 1054 / 1171, 12 931 / 950, 16
+// 880 / 852, 24 837 / 755; 4096 x 512 (19 M) 8 1052 / 1783, 24 845 / 1084;
+// 4096^2 (34 M) 16 5837 / 7405, 50 5481 / 5596; 5000^2 (50 M) 50 8237 / 9082) ...
+constexpr long long overlap_from(long long elems) {
+    return elems >> 19 > 16 ? elems >> 19 : 16;
+}
+// ... and an LP with fewer rows or columns than this, which takes few pivots (us a
+// solve in turn / overlapped: 5000 x 2 1 pivot 41 / 223, x 16 12 pivots 111 / 258,
+// x 64 301 / 444, x 128 410 / 543; 2000 x 64 176 / 186, x 128 177 / 183, x 300 268 /
+// 258; 3000 x 128 175 / 187, dual 271 / 254).
+constexpr int kOverlapSide = 64;
+
+// Wide LPs (n > 4 m), where no column is left out: whether the panel kernel takes
+// one.  Its G CTAs split the panels by rows, `rows` at most each, and every CTA
+// reads the pending rows whole, so it loses to the kernels that split the columns
+// where the tableau is long, more so where the rows do not divide evenly, and
+// where a last panel has few rows to work on.  Measured on 152 CTAs, us per pivot,
+// this kernel / the column split (primal rule unless said): 64 x 6000 9.0 / 9.5, x
+// 12000 10.1 / 8.7; 150 x 8000 8.4 / 9.5, x 22000 13.5 / 11.8; 200 x 14000 12.9 /
+// 10.0; 300 x 8000 9.1 / 10.3, x 22000 20.0 / 17.9; 310 x 10000 12.6 / 11.3; 600 x
+// 14000 19.5 / 22.3; 800 x 22000 41.2 / 38.7; 1100 x 17000 40.4 / 41.9, x 22000
+// 52.3 / 51.4; 3 x 8000, dual, its one pivot 39 / 20; in turn 160 x 6000, dual, 10.3
+// / 9.2, 200 x 4000 9.0 / 9.2.
+bool panel_takes_wide(long long m, long long N, long long G, bool overlap) {
+    const long long rows = (m + G - 1) / G, W = (N + G - 1) / G;
+    return m >= 16 && (W - 40) * rows * G * G <= 16 * m * m &&
+           (overlap || rows == 1 || 5 * m >= 3 * rows * G);
+}
 
 struct lp_handle {
     lp_options opt;
@@ -402,9 +433,8 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     // where its shared memory and its workspace fit (a workspace above 64 MB
     // only when the tableau is at least twice as large), with overlapped
     // panels where they pay and the second buffer can be had.  Wide LPs from
-    // 2^20 elements, where no column is left out and a CTA's few rows split
-    // unevenly, only with overlapped panels (512 x 4096: 8.6 us per pivot; in
-    // turn 10.9, the two-pivot kernel 10.1).
+    // 2^20 elements only with overlapped panels (512 x 4096: 8.6 us per pivot;
+    // in turn 10.9, the two-pivot kernel 10.1).
     const int pdrop = h->opt.zero_skip == 2 || (h->opt.zero_skip == 1 && 4ll * m >= n);
     auto panel_shape = [&](int rule, bool ov) {
         return choose_panel_shape(h->prec, M, N, h->sms, h->opt.ctas, rule, pdrop, ov);
@@ -415,8 +445,11 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     bool panel = h->opt.pipeline == 1 && psh.pipe == 4 &&
                  (pws <= (64ull << 20) || 2 * pws <= tbytes);
     bool overlap = panel && h->prec == PREC_FP64 && elems >= kOverlapElems &&
-                   elems < kOverlapPerCta * psh.ctas && panel_shape((int)sense, true).pipe == 5;
-    panel = panel && (4ll * m >= n || elems < (1ll << 20) || overlap);
+                   elems < kOverlapPerCta * psh.ctas && h->opt.max_iters >= overlap_from(elems) &&
+                   std::min(m, n) >= kOverlapSide && panel_shape((int)sense, true).pipe == 5;
+    panel = panel && (4ll * m >= n || ((elems < (1ll << 20) || overlap) &&
+                                       panel_takes_wide(m, N, psh.ctas, overlap)));
+    overlap = overlap && panel;
     if (panel && h->region) {
         // (what the buffers below take besides the inputs, with slack)
         size_t need = tbytes + pws + (size_t)(m + n) * 16 +
@@ -635,7 +668,7 @@ namespace {
 // The words a pivot launch wants zeroed: the synchronisation block, and the
 // records of the panel kernel.
 size_t bar_bytes(const PivotShape &sh) {
-    return (kBarWords + (sh.pipe >= 4 ? kPanelRecWords : 0)) * sizeof(unsigned);
+    return (kBarWords + (sh.pipe >= 4 ? panel_rec_words(sh.ctas) : 0)) * sizeof(unsigned);
 }
 
 // Start the wall-clock limit of a solve: lower the abort word (no kernel of
@@ -661,6 +694,14 @@ PivotShape timed(const lp_handle *h, PivotShape sh) {
             1, std::chrono::duration_cast<std::chrono::nanoseconds>(left).count());
     }
     return sh;
+}
+
+// The shape of a launch of at most `budget` pivots.
+PivotShape launch_shape(const lp_handle *h, const PivotShape &sh, long long budget) {
+    if (sh.pipe == 5 && budget < overlap_from((long long)h->M * h->P))
+        return timed(h, choose_panel_shape(h->prec, h->M, h->N, h->sms, h->opt.ctas, sh.dual,
+                                           sh.drop, false));
+    return timed(h, sh);
 }
 
 // Wait for the handle's stream.  Under a wall-clock limit the host polls the
@@ -820,10 +861,10 @@ lp_err solve_fp32(lp_handle *h) {
         const long long stride = sh.scratch_stride;
         CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, scratch_stride), &stride,
                                     sizeof stride, cudaMemcpyHostToDevice, s));
-        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape_alt), s));
+        CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(sh), s));
         CUDA_TRY(h, cudaEventRecord(h->ev0, s));
-        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, sh), h->opt.spin_timeout_cycles, budget,
-                                 s));
+        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, launch_shape(h, sh, budget),
+                                 h->opt.spin_timeout_cycles, budget, s));
         CUDA_TRY(h, cudaEventRecord(h->ev1, s));
         CUDA_TRY(h, cudaMemcpyAsync(h->pdesc, h->ddesc, sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(h, wait_stream(h));
@@ -928,7 +969,7 @@ lp_err lp_solve_async(lp_handle *h) {
         // host waits for its end to choose what follows.
         const long long before = h->pdesc->iters;
         CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
-        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, h->shape_alt),
+        CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, launch_shape(h, h->shape_alt, budget),
                                  h->opt.spin_timeout_cycles, budget, s));
         CUDA_TRY(h, cudaMemcpyAsync(h->pdesc, h->ddesc, sizeof(LpDesc), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(h, wait_stream(h));
@@ -960,8 +1001,8 @@ lp_err lp_solve_async(lp_handle *h) {
         }
     }
     CUDA_TRY(h, cudaMemsetAsync(h->dbar, 0, bar_bytes(h->shape), s));
-    CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, timed(h, h->shape), h->opt.spin_timeout_cycles,
-                             budget, s));
+    CUDA_TRY(h, launch_pivot(h->prec, h->ddesc, launch_shape(h, h->shape, budget),
+                             h->opt.spin_timeout_cycles, budget, s));
     CUDA_TRY(h, cudaEventRecord(h->ev1, s));
     CUDA_TRY(h, launch_extract(h->prec, h->ddesc, h->dT, h->dbasis, h->m, h->n, h->P, h->sense,
                                h->dx, h->dy, h->dobj, s));

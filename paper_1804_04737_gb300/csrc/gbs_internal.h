@@ -128,7 +128,8 @@ constexpr int kPanelOverlapK = 8;  // and as many of the panel being applied
 static_assert(2 * kPanelOverlapK == kPanelK, "the overlapped panels use the same slots");
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxCtas = 192;
-constexpr int kPanelRecWords = 2 * kPanelMaxCtas * 32;
+constexpr int panel_rec_words(int ctas) { return 2 * ctas * 32; }
+constexpr int kPanelRecWords = panel_rec_words(kPanelMaxCtas);
 
 struct InputStats {
     unsigned long long amax_bits, bmax_bits, cmax_bits;  // bit patterns of max |.|
