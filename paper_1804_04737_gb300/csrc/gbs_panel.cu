@@ -469,17 +469,17 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
         }
         for (int w = tid; w < nwords; w += B) bb[w] = 0;
         // the padding of the last vector of the pending rows (other CTAs read
-        // it once this CTA's records are out)
+        // it once a record or the barrier has announced the rows)
         if (g == 0 && tid < NS)
             for (int j = N; j < nvec * VW; ++j) __stcg(PR + tid * P + j, (T)0);
-        __threadfence();
+        const int bas0 = tid < m ? __ldcg(d->basis + tid) : -1;
         if (tid == 0) {
             s_fail[0] = s_fail[1] = 0;
             s_nflag = 0;
         }
         cta_sync();
         for (int i = tid; i < m; i += B) {
-            const int j = __ldcg(d->basis + i);
+            const int j = i == tid ? bas0 : __ldcg(d->basis + i);
             atomicOr(&bb[j >> 5], 1u << (j & 31));
         }
         cta_sync();
@@ -671,9 +671,10 @@ __device__ __forceinline__ void panel_solve(LpDesc *__restrict__ d, int G, int g
             }
         }
         // other CTAs read these rows after this CTA's next record: whichever
-        // thread publishes it, its fence follows every thread's writes
+        // thread publishes it, its fence follows every thread's writes (a launch
+        // that ends publishes no more)
         sync();
-        __threadfence();
+        if (OV || status == ST_RUNNING) __threadfence();
     };
     // The pending pivots of a full or last panel, in place (not OV).
     auto apply_panel = [&](int kk) {
