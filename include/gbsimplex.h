@@ -198,7 +198,8 @@ typedef struct {
                                 FP32 body does not build up; 0 = only the rhs,
                                 the duals and the objective row.  Batches do
                                 the latter.                                     */
-    int zero_skip;           /* panel kernel (pipeline 1): 1 (default, where
+    int zero_skip;           /* single-LP solves (batches: always as 1 at any
+                                shape).  Panel kernel (pipeline 1): 1 (default, where
                                 m >= n / 4) and 2 = a panel leaves out the
                                 columns that are basic throughout it, whose
                                 entries in its pivot rows are zeros; 0 = it

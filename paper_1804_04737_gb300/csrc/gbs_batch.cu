@@ -250,7 +250,7 @@ struct BatchFp32 {
     int2 *h_items, *d_items;
     unsigned *d_queue;
     unsigned char *d_bar;
-    int ctas, threads, use_smem, sms, panel, drop;
+    int ctas, threads, use_smem, sms, panel;
     size_t smem, bar_bytes;
     const lp_options *opt;
     cudaStream_t s;
@@ -309,7 +309,7 @@ lp_err solve_batch_fp32(const BatchFp32 &f, lp_status *fin, double *kernel_ms) {
         B_TRY(cudaEventRecord(e0, s));
         if (f.panel)
             B_TRY(launch_panel_batch(PREC_FP32, f.d_desc, f.d_items, nitems, f.d_queue, f.ctas,
-                                     f.smem, f.opt->spin_timeout_cycles, budget, f.drop, s));
+                                     f.smem, f.opt->spin_timeout_cycles, budget, s));
         else
             B_TRY(launch_batch(PREC_FP32, f.d_desc, f.d_items, nitems, f.d_queue, f.ctas,
                                f.threads, f.smem, f.use_smem, f.opt->spin_timeout_cycles, budget,
@@ -436,7 +436,6 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     // The panel kernel takes the batch where every LP's slices fit its shared
     // memory: half an SM's, two CTAs per SM, on as many CTAs per LP as that
     // needs.  The kernel that updates the tableau every pivot is for the rest.
-    const int drop = o.zero_skip != 0;
     bool panel = true;
     for (int k = 0; k < count && panel; ++k)
         panel = panel_smem(prec, m[k], n[k] + m[k] + 1, std::min(sms, kPanelMaxCtas),
@@ -715,7 +714,6 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         f.use_smem = use_smem;
         f.sms = sms;
         f.panel = panel;
-        f.drop = drop;
         f.bar_bytes = bar_bytes;
         f.opt = &o;
         f.s = s;
@@ -754,7 +752,7 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     if (panel)
         B_TRY(launch_panel_batch(prec, d_desc, reinterpret_cast<const int2 *>(D + o_items),
                                  (int)items.size(), reinterpret_cast<unsigned *>(D + o_queue), ctas,
-                                 smem, o.spin_timeout_cycles, o.max_iters, drop, s));
+                                 smem, o.spin_timeout_cycles, o.max_iters, s));
     else
         B_TRY(launch_batch(prec, d_desc, reinterpret_cast<const int2 *>(D + o_items),
                            (int)items.size(), reinterpret_cast<unsigned *>(D + o_queue), ctas,

@@ -186,10 +186,11 @@ size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K);
 size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap = false);
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s);
-// The same over a batch's work items, panels of kPanelBatchK.
+// The same over a batch's work items, panels of kPanelBatchK that leave out the
+// columns that stay basic.
 cudaError_t launch_panel_batch(int prec, LpDesc *descs, const int2 *items, int nitems,
                                unsigned *queue, int ctas, size_t smem, long long spin_limit,
-                               long long budget, int drop, cudaStream_t s);
+                               long long budget, cudaStream_t s);
 int max_coresident_panel_batch_ctas(int prec, size_t smem, int sms);
 cudaError_t launch_extract(int prec, const LpDesc *d_desc, const void *T, const int *basis,
                            int m, int n, long long P, int sense, double *x, double *y,

@@ -1,0 +1,48 @@
+"""GPU: the kernels a batch may take give the oracle's bits, whichever takes it.
+
+lp_batch_stats tells which it was: the panel kernel has CTAs of 256 threads, the
+kernel that updates the tableau every pivot the threads asked for (512).
+"""
+import os
+
+import pytest
+
+import oracle
+from paper_1804_04737_gb300 import capi, lpgen
+from paper_1804_04737_gb300.build import build_library
+from test_gpu_batch import _check_against_oracle
+
+pytestmark = pytest.mark.gpu
+
+PANEL, EVERY_PIVOT = 256, 512
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_library()
+    capi.load_library()
+    oracle.set_threads(os.cpu_count() or 1)
+    yield
+    oracle.set_threads(1)
+
+
+def _lps(shapes, dual=False):
+    lps = []
+    for k, (m, n) in enumerate(shapes):
+        if dual:
+            lps.append((*lpgen.dual_of(*lpgen.dense_lp(n, m, seed=k)), capi.LP_MIN_GE))
+        else:
+            lps.append((*lpgen.dense_lp(m, n, seed=k), capi.LP_MAX_LE))
+    return lps
+
+
+def _solve(lps, kernel, **opts):
+    _check_against_oracle(lps, capi.lp_solve_batch(lps, capi.lp_options_default(**opts), want_xy=True))
+    assert capi.lp_batch_stats()[3] == kernel
+
+
+@pytest.mark.parametrize("zero_skip", [0, 1, 2])
+@pytest.mark.parametrize("dual", [False, True])
+def test_zero_skip(dual, zero_skip):
+    """Batches leave out the columns that stay basic whatever is asked."""
+    _solve(_lps([(60, 50), (9, 30), (200, 40), (33, 17)], dual), PANEL, zero_skip=zero_skip)
