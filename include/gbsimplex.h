@@ -329,10 +329,11 @@ lp_err lp_kernel_time(lp_handle *h, double *ms, int *launches);
  * LP_FP32_REINV the tableaus are FP32 and every LP is reinverted in FP64
  * (batched) every reinv_k pivots and at termination, as in the single-LP FP32
  * mode (b >= 0 and c >= 0 required); each result then equals that LP's solo
- * FP32 solve.  CTAs have 256 threads; opt->threads (at most 512) is for batches
- * with an LP whose slices do not fit the panel kernel's shared memory, which
- * the kernel of pipeline 0 takes; device memory is pooled
- * per device between calls.
+ * FP32 solve.  The panel kernel's CTAs have 256 threads; opt->threads (at most
+ * 512) is for the batches that the kernel of pipeline 0 takes: those with an LP
+ * whose slices do not fit the panel kernel's shared memory, and those of few
+ * CTAs and mostly of wide LPs (n > 4 m) with long rows.  Device memory is
+ * pooled per device between calls.
  * Blocking.  Errors as lp_load (the message names the LP), in
  * lp_last_error(NULL). */
 lp_err lp_solve_batch(int count, const int *m, const int *n, const double *const *A,

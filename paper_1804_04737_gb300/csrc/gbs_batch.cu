@@ -435,7 +435,14 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
 
     // The panel kernel takes the batch where every LP's slices fit its shared
     // memory: half an SM's, two CTAs per SM, on as many CTAs per LP as that
-    // needs.  The kernel that updates the tableau every pivot is for the rest.
+    // needs.  The kernel that updates the tableau every pivot is for the rest,
+    // and for batches of fewer than two CTAs per SM whose tableaus are mostly
+    // those of wide LPs (n > 4 m) with long rows: no column is left out of those,
+    // and one CTA of 256 threads alone on its SM updates them at two thirds of the
+    // rate of one of 512.  Measured, us, panels / every pivot: 1 LP of 300 x 3000 5375 /
+    // 3403, 6 of 100 x 6000 2533 / 1496, 60 of 10 x 2000 656 / 519 (600 of them 1.5
+    // times as fast in panels), 60 of 40 x 400 dual 253 / 241 (primal 1.2 times);
+    // FP32 rounds only with few rows: 1 of 5 x 12000 226 / 146, of 10 x 2000 1.06.
     bool panel = true;
     for (int k = 0; k < count && panel; ++k)
         panel = panel_smem(prec, m[k], n[k] + m[k] + 1, std::min(sms, kPanelMaxCtas),
@@ -445,33 +452,51 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     std::vector<int> M(count), N(count), G(count), W(count), sv(count);
     std::vector<long long> P(count);
     size_t smem_max = 0, sprow_max = 0;
-    for (int k = 0; k < count; ++k) {
-        M[k] = m[k] + 1;
-        N[k] = n[k] + m[k] + 1;
-        P[k] = pitch_for(N[k]);
-        sv[k] = sense ? sense[k] : 0;
-        if (panel) {
+    auto shapes = [&]() {
+        smem_max = sprow_max = 0;
+        for (int k = 0; k < count; ++k) {
+            M[k] = m[k] + 1;
+            N[k] = n[k] + m[k] + 1;
+            P[k] = pitch_for(N[k]);
+            sv[k] = sense ? sense[k] : 0;
+            if (panel) {
+                long long g = ((long long)M[k] * P[k] + gelems - 1) / gelems;
+                g = std::max<long long>(1, std::min<long long>(g, std::min(std::min(sms, kPanelMaxCtas), N[k])));
+                while (panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK) > kPanelBatchSmem) ++g;
+                G[k] = (int)g;
+                W[k] = 0;
+                smem_max = std::max(smem_max, panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK));
+                continue;
+            }
+            const long long gmin = (P[k] + (long long)threads * vw - 1) / ((long long)threads * vw);
             long long g = ((long long)M[k] * P[k] + gelems - 1) / gelems;
-            g = std::max<long long>(1, std::min<long long>(g, std::min(std::min(sms, kPanelMaxCtas), N[k])));
-            while (panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK) > kPanelBatchSmem) ++g;
-            G[k] = (int)g;
-            W[k] = 0;
-            smem_max = std::max(smem_max, panel_smem(prec, m[k], N[k], (int)g, kPanelBatchK));
-            continue;
+            g = std::min<long long>(g, std::min<long long>(sms, P[k] / sector));
+            g = std::max<long long>(g, gmin);
+            long long w = (P[k] + g - 1) / g;
+            w = (w + sector - 1) / sector * sector;
+            W[k] = (int)w;
+            G[k] = (int)((P[k] + w - 1) / w);
+            const size_t sprow = ((size_t)w * esz + 15) & ~(size_t)15;
+            const size_t scol = ((size_t)M[k] * esz + 15) & ~(size_t)15;
+            const size_t sr = (size_t)(sv[k] == 0 && !fp32 ? M[k] : N[k]) * sizeof(double);
+            smem_max = std::max(smem_max, sprow + scol + sr);
+            sprow_max = std::max(sprow_max, sprow);
         }
-        const long long gmin = (P[k] + (long long)threads * vw - 1) / ((long long)threads * vw);
-        long long g = ((long long)M[k] * P[k] + gelems - 1) / gelems;
-        g = std::min<long long>(g, std::min<long long>(sms, P[k] / sector));
-        g = std::max<long long>(g, gmin);
-        long long w = (P[k] + g - 1) / g;
-        w = (w + sector - 1) / sector * sector;
-        W[k] = (int)w;
-        G[k] = (int)((P[k] + w - 1) / w);
-        const size_t sprow = ((size_t)w * esz + 15) & ~(size_t)15;
-        const size_t scol = ((size_t)M[k] * esz + 15) & ~(size_t)15;
-        const size_t sr = (size_t)(sv[k] == 0 && !fp32 ? M[k] : N[k]) * sizeof(double);
-        smem_max = std::max(smem_max, sprow + scol + sr);
-        sprow_max = std::max(sprow_max, sprow);
+    };
+    shapes();
+    if (panel) {
+        long long ctas_all = 0, elems = 0, wide = 0;
+        for (int k = 0; k < count; ++k) {
+            const long long e = (long long)M[k] * P[k];
+            ctas_all += G[k];
+            elems += e;
+            const int longest = !fp32 ? (sv[k] ? 400 : 1000) : 4000;
+            if (n[k] > 4ll * m[k] && N[k] > longest && (!fp32 || m[k] < 16)) wide += e;
+        }
+        if (ctas_all < 2 * sms && 2 * wide > elems) {
+            panel = false;
+            shapes();
+        }
     }
     if (panel) threads = kPanelThreads;
     const int use_smem = smem_max <= 200 * 1024 ? 1 : 0;

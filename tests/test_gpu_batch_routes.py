@@ -46,3 +46,15 @@ def _solve(lps, kernel, **opts):
 def test_zero_skip(dual, zero_skip):
     """Batches leave out the columns that stay basic whatever is asked."""
     _solve(_lps([(60, 50), (9, 30), (200, 40), (33, 17)], dual), PANEL, zero_skip=zero_skip)
+
+
+@pytest.mark.parametrize("dual", [False, True])
+def test_few_wide_lps(dual):
+    """Most of the tableau elements in wide LPs with long rows, fewer than two
+    CTAs per SM: the column split; otherwise panels."""
+    wide, square = (30, 1500), (150, 140)
+    _solve(_lps([wide, (40, 40), (9, 1200)], dual), EVERY_PIVOT)
+    _solve(_lps([wide, square, square, square], dual), PANEL)
+    _solve(_lps([(30, 350), (6, 300)], dual), PANEL)
+    _solve(_lps([(30, 450)], dual), EVERY_PIVOT if dual else PANEL)
+    _solve(_lps([(12, 1100)] * 320, dual), PANEL)
