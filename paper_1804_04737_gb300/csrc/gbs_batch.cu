@@ -392,13 +392,13 @@ lp_err solve_batch_fp32(const BatchFp32 &f, lp_status *fin, double *kernel_ms) {
     return LP_OK;
 }
 
-}  // namespace
-
-extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const double *const *A,
-                                 const double *const *b, const double *const *c,
-                                 const int *sense, const lp_options *opt, double *obj,
-                                 lp_status *status, long long *iters, double *const *x,
-                                 double *const *y) {
+// The batch (lp_solve_batch).  With no_room it may take the panel kernel, and sets
+// *no_room and does nothing where the device has no room for that kernel's
+// workspace beside the tableaus.
+lp_err solve_batch(int count, const int *m, const int *n, const double *const *A,
+                   const double *const *b, const double *const *c, const int *sense,
+                   const lp_options *opt, double *obj, lp_status *status, long long *iters,
+                   double *const *x, double *const *y, bool *no_room) {
     if (count < 1 || !m || !n || !A || !b || !c)
         return bfail(LP_ERR_INVALID_ARG, "lp_solve_batch: need count >= 1 and non-NULL arrays");
     lp_options o;
@@ -443,7 +443,7 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     // 3403, 6 of 100 x 6000 2533 / 1496, 60 of 10 x 2000 656 / 519 (600 of them 1.5
     // times as fast in panels), 60 of 40 x 400 dual 253 / 241 (primal 1.2 times);
     // FP32 rounds only with few rows: 1 of 5 x 12000 226 / 146, of 10 x 2000 1.06.
-    bool panel = true;
+    bool panel = no_room != nullptr;
     for (int k = 0; k < count && panel; ++k)
         panel = panel_smem(prec, m[k], n[k] + m[k] + 1, std::min(sms, kPanelMaxCtas),
                            kPanelBatchK) <= kPanelBatchSmem;
@@ -569,7 +569,13 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
     Pool &pool = g_pool[o.device];
     std::lock_guard<std::mutex> lock(pool.mu);
     void *dv = nullptr, *pv = nullptr;
-    B_TRY(pool_dev(pool, dev_total, &dv));
+    const cudaError_t pe = pool_dev(pool, dev_total, &dv);
+    if (pe == cudaErrorMemoryAllocation && panel) {
+        cudaGetLastError();
+        *no_room = true;
+        return LP_ERR_OOM;
+    }
+    B_TRY(pe);
     B_TRY(pool_pin(pool, pin_total, &pv));
     unsigned char *D = static_cast<unsigned char *>(dv), *H = static_cast<unsigned char *>(pv);
     InputStats *h_stats = reinterpret_cast<InputStats *>(H + meta_bytes);
@@ -815,6 +821,20 @@ extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const do
         g_last.max_group = max_group;
     }
     return LP_OK;
+}
+
+}  // namespace
+
+extern "C" lp_err lp_solve_batch(int count, const int *m, const int *n, const double *const *A,
+                                 const double *const *b, const double *const *c,
+                                 const int *sense, const lp_options *opt, double *obj,
+                                 lp_status *status, long long *iters, double *const *x,
+                                 double *const *y) {
+    bool no_room = false;
+    lp_err e = solve_batch(count, m, n, A, b, c, sense, opt, obj, status, iters, x, y, &no_room);
+    if (no_room)
+        e = solve_batch(count, m, n, A, b, c, sense, opt, obj, status, iters, x, y, nullptr);
+    return e;
 }
 
 extern "C" lp_err lp_batch_stats(double *kernel_ms, long long *pivots, int *ctas, int *threads,

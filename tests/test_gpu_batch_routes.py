@@ -4,6 +4,8 @@ lp_batch_stats tells which it was: the panel kernel has CTAs of 256 threads, the
 kernel that updates the tableau every pivot the threads asked for (512).
 """
 import os
+import subprocess
+import sys
 
 import pytest
 
@@ -58,3 +60,35 @@ def test_few_wide_lps(dual):
     _solve(_lps([(30, 350), (6, 300)], dual), PANEL)
     _solve(_lps([(30, 450)], dual), EVERY_PIVOT if dual else PANEL)
     _solve(_lps([(12, 1100)] * 320, dual), PANEL)
+
+
+NO_ROOM = """
+import sys
+sys.path[:0] = [%r, %r]
+import numpy as np
+import torch
+from paper_1804_04737_gb300 import capi, lpgen
+from test_gpu_batch import _check_against_oracle
+few = [(*lpgen.dense_lp(8, 8, seed=1), capi.LP_MAX_LE)]
+capi.lp_solve_batch(few)
+lps = [(*lpgen.dense_lp(1, 4000, seed=k), capi.LP_MAX_LE) for k in range(40)] * 100
+held = torch.empty(torch.cuda.mem_get_info()[0] - (1800 << 20), dtype=torch.uint8, device="cuda")
+obj, st, it, xs, ys = capi.lp_solve_batch(lps, want_xy=True)
+print("threads", capi.lp_batch_stats()[3])
+_check_against_oracle(lps[:40], (obj[:40], st[:40], it[:40], xs[:40], ys[:40]))
+assert all(np.array_equal(xs[k], xs[k %% 40]) for k in range(len(lps)))
+del held
+torch.cuda.empty_cache()
+capi.lp_solve_batch(lps)
+print("threads", capi.lp_batch_stats()[3])
+"""
+
+
+def test_no_room_for_the_panels():
+    """4000 LPs of 1 x 4000 take 0.5 GB, and 3 GB more for the pending rows and
+    columns of the panel kernel: with 1.8 GB free they run without it."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", NO_ROOM % (os.path.dirname(here), here)], capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.split() == ["threads", str(EVERY_PIVOT), "threads", str(PANEL)]
