@@ -463,6 +463,9 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
         overlap = overlap && room >= need + tbytes + 256;
         panel = room >= need;
     }
+    // (the tableau before what a solve can do without; from a range, whose room
+    // was looked at, after it)
+    if (!h->region) CUDA_TRY(h, grow_bytes(h, &h->dT, &h->cap_T, tbytes));
     if (panel && grow_bytes(h, &h->dpanel, &h->cap_panel, pws) != cudaSuccess) {
         cudaGetLastError();
         panel = false;
