@@ -709,6 +709,8 @@ lp_err solve_batch(int count, const int *m, const int *n, const double *const *A
     B_TRY(cudaMemcpyAsync(d_desc, h_desc, count * sizeof(LpDesc), cudaMemcpyHostToDevice, s));
     B_TRY(cudaMemsetAsync(D + o_bar, 0, bar_bytes, s));
     B_TRY(cudaMemsetAsync(D + o_queue, 0, sizeof(unsigned), s));
+    // (the panel kernel's workspaces: what the arena held there could be a live tag)
+    if (panel) B_TRY(cudaMemsetAsync(D + o_part, 0, part_total, s));
     if (fp32)
         batch_build_kernel<float><<<dim3(16, count), 256, 0, s>>>(
             ba, d_in, D + o_T, reinterpret_cast<int *const *>(D + o_bptr));

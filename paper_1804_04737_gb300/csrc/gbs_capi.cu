@@ -115,6 +115,7 @@ struct lp_handle {
     size_t cap_colx = 0;
     void *dpanel = nullptr;                     // panel kernel: pending columns and rows
     size_t cap_panel = 0;
+    int panel_m = 0, panel_N = 0, panel_ctas = 0;  // the layout its tagged values were cleared for
     int *dbasis = nullptr;
     size_t cap_basis = 0;
     void *dscratch = nullptr;
@@ -466,9 +467,20 @@ lp_err lp_load(lp_handle *h, int m, int n, const double *A, const double *b, con
     // (the tableau before what a solve can do without; from a range, whose room
     // was looked at, after it)
     if (!h->region) CUDA_TRY(h, grow_bytes(h, &h->dT, &h->cap_T, tbytes));
-    if (panel && grow_bytes(h, &h->dpanel, &h->cap_panel, pws) != cudaSuccess) {
-        cudaGetLastError();
-        panel = false;
+    if (panel) {
+        const size_t had = h->cap_panel;
+        if (grow_bytes(h, &h->dpanel, &h->cap_panel, pws) != cudaSuccess) {
+            cudaGetLastError();
+            panel = false;
+        } else if (h->region || h->cap_panel != had || h->panel_m != m || h->panel_N != N ||
+                   h->panel_ctas != psh.ctas) {
+            // where a tagged value will lie may hold anything, a live tag too;
+            // from here on it holds tags of earlier loads alone
+            CUDA_TRY(h, cudaMemsetAsync(h->dpanel, 0, panel_tagged(m, N, psh.ctas, kPanelK), h->stream));
+            h->panel_m = m;
+            h->panel_N = N;
+            h->panel_ctas = psh.ctas;
+        }
     }
     if (overlap && (!panel || grow_bytes(h, &h->dT2, &h->cap_T2, tbytes) != cudaSuccess)) {
         if (panel) cudaGetLastError();

@@ -89,7 +89,8 @@ struct LpDesc {
 };
 
 // A number no other load or batched launch of this process has: the panel
-// kernels' tags differ, whichever handle's memory they meet.
+// kernels' tags differ, whichever handle's memory they meet.  (Memory that held
+// something else is cleared first: any bits could be a tag.)
 unsigned panel_nonce();
 
 // Launch shape of the persistent pivot kernel for one LP.
@@ -183,6 +184,8 @@ cudaError_t launch_pivot_pipe(int prec, LpDesc *d_desc, const PivotShape &sh,
 PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dual, int drop,
                               bool overlap);
 size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K);
+// Its first bytes, which hold the values with tags.
+size_t panel_tagged(int m, long long N, int G, int K);
 size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap = false);
 cudaError_t launch_panel(int prec, LpDesc *d_desc, const PivotShape &sh, long long spin_limit,
                          long long budget, cudaStream_t s);

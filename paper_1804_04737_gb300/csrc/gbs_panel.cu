@@ -1653,9 +1653,11 @@ PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dua
 
 size_t panel_workspace(int prec, int m, long long N, long long P, int G, int K) {
     const size_t esz = prec == PREC_FP64 ? 8 : 4;
-    const size_t tagged =
-        G > 1 ? (size_t)K * (size_t)(tag_pitch(m) + tag_pitch(N)) * 16 + 256 * (size_t)G : 0;
-    return tagged + (size_t)K * (size_t)P * esz + (size_t)m;
+    return panel_tagged(m, N, G, K) + (size_t)K * (size_t)P * esz + (size_t)m;
+}
+
+size_t panel_tagged(int m, long long N, int G, int K) {
+    return G > 1 ? (size_t)K * (size_t)(tag_pitch(m) + tag_pitch(N)) * 16 + 256 * (size_t)G : 0;
 }
 
 size_t panel_smem(int prec, int m, int N, int G, int K, bool overlap) {
