@@ -122,7 +122,9 @@ typedef struct {
     double eps_p;            /* <= 0: 1e-9 * max(1, max|A|)                       */
     double eps_r;            /* <= 0: 1e-9 * max(1, max|b|)                       */
     int bland_after;         /* consecutive zero-ratio pivots before Bland's rule */
-    int threads;             /* threads per CTA of the pivot kernel, 0 = auto     */
+    int threads;             /* threads per CTA of the pivot kernel, 0 = auto; the
+                                panel kernel (pipeline, below) has 256, or 512
+                                with a second buffer, whatever is asked       */
     long long spin_timeout_cycles; /* device wait limit (SM clock cycles)        */
     void *cuda_stream;       /* cudaStream_t to run on; NULL = library's own      */
     int device;              /* CUDA device ordinal                               */
@@ -342,7 +344,8 @@ lp_err lp_solve_batch(int count, const int *m, const int *n, const double *const
                       double *const *x, double *const *y);
 
 /* Autotuner for lp_solve_batch: times every candidate launch shape
- * (group_elems in {16K, 64K, 256K, 1M} x threads in {256, 512}) on this
+ * (group_elems in {16K, 64K, 256K, 1M} x threads in {256, 512}, once where the
+ * panel kernel takes the batch, whose CTAs have 256) on this
  * batch, best of two solves each, and returns in *best a copy of *opt (NULL:
  * defaults) with the fastest group_elems and threads.  With a non-NULL
  * cache_path the choice is looked up in / appended to that text file, keyed

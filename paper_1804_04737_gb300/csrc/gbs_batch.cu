@@ -852,9 +852,10 @@ extern "C" lp_err lp_batch_stats(double *kernel_ms, long long *pivots, int *ctas
 
 // ------------------------------------------------------------- autotuner --
 //
-// Picks the batched launch shape (tableau elements per CTA of a group, CTA
-// size) for a batch by timing every candidate on the batch itself (the best
-// of two solves each, batched pivot kernel time).  Results are cached in a
+// Picks the batched launch shape (tableau elements per CTA of a group, and the
+// CTA size where the batch's kernel has a choice) for a batch by timing every
+// candidate on the batch itself (the best of two solves each, batched pivot
+// kernel time).  Results are cached in a
 // text file, one line "key group_elems threads kernel_ms" per batch
 // signature (count and a hash of the sorted shapes), so a serving process
 // tunes once per workload mix.
@@ -915,7 +916,7 @@ extern "C" lp_err lp_batch_autotune(int count, const int *m, const int *n,
         return LP_OK;
     }
     static const long long kElems[] = {16384, 65536, 262144, 1048576};
-    static const int kThreads[] = {256, 512};
+    static const int kThreads[] = {512, 256};
     double best_ms = 1e300;
     for (long long e : kElems)
         for (int t : kThreads) {
@@ -923,19 +924,22 @@ extern "C" lp_err lp_batch_autotune(int count, const int *m, const int *n,
             trial.group_elems = e;
             trial.threads = t;
             double ms = 1e300;
+            int ran = 0;
             for (int rep = 0; rep < 2; ++rep) {
                 lp_err r = lp_solve_batch(count, m, n, A, b, c, sense, &trial, nullptr, nullptr,
                                           nullptr, nullptr, nullptr);
                 if (r != LP_OK) return r;
                 double k_ms = 0.0;
-                lp_batch_stats(&k_ms, nullptr, nullptr, nullptr, nullptr);
+                lp_batch_stats(&k_ms, nullptr, nullptr, &ran, nullptr);
                 ms = std::min(ms, k_ms);
             }
             if (ms < best_ms) {
                 best_ms = ms;
                 ge = e;
-                th = t;
+                th = ran;
             }
+            // the panel kernel's CTAs have one size, whatever is asked for
+            if (ran != t) break;
         }
     *best = o;
     best->group_elems = ge;

@@ -92,3 +92,15 @@ def test_no_room_for_the_panels():
                        text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     assert r.stdout.split() == ["threads", str(EVERY_PIVOT), "threads", str(PANEL)]
+
+
+@pytest.mark.parametrize("kernel,shapes", [(PANEL, [(60, 50), (9, 30), (200, 40)]), (EVERY_PIVOT, [(2, 1500)] * 3)])
+def test_autotune_on_either_kernel(kernel, shapes):
+    """The choice names the CTA size it was timed with: the panel kernel's one
+    size, or one of two."""
+    lps = _lps(shapes)
+    _solve(lps, kernel)
+    best = capi.lp_batch_autotune(lps)
+    assert best.threads in ((256,) if kernel == PANEL else (256, 512))
+    _check_against_oracle(lps, capi.lp_solve_batch(lps, best, want_xy=True))
+    assert capi.lp_batch_stats()[3] == best.threads
