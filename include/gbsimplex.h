@@ -349,7 +349,7 @@ lp_err lp_solve_batch(int count, const int *m, const int *n, const double *const
  * batch, best of two solves each, and returns in *best a copy of *opt (NULL:
  * defaults) with the fastest group_elems and threads.  With a non-NULL
  * cache_path the choice is looked up in / appended to that text file, keyed
- * by the batch size and a hash of its sorted shapes. */
+ * by the kernel, the batch size and a hash of its sorted shapes. */
 lp_err lp_batch_autotune(int count, const int *m, const int *n, const double *const *A,
                          const double *const *b, const double *const *c, const int *sense,
                          const lp_options *opt, const char *cache_path, lp_options *best);

@@ -392,6 +392,17 @@ lp_err solve_batch_fp32(const BatchFp32 &f, lp_status *fin, double *kernel_ms) {
     return LP_OK;
 }
 
+// Whether every LP's slices fit the panel kernel's shared memory.
+bool panel_fits(int count, const int *m, const int *n, int prec, int sms) {
+    for (int k = 0; k < count; ++k) {
+        const long long N = (long long)n[k] + m[k] + 1;
+        if (m[k] < 1 || n[k] < 1 || N > 0x7fffffffll - 64 ||
+            panel_smem(prec, m[k], (int)N, std::min(sms, kPanelMaxCtas), kPanelBatchK) > kPanelBatchSmem)
+            return false;
+    }
+    return true;
+}
+
 // The batch (lp_solve_batch).  With no_room it may take the panel kernel, and sets
 // *no_room and does nothing where the device has no room for that kernel's
 // workspace beside the tableaus.
@@ -443,10 +454,7 @@ lp_err solve_batch(int count, const int *m, const int *n, const double *const *A
     // 3403, 6 of 100 x 6000 2533 / 1496, 60 of 10 x 2000 656 / 519 (600 of them 1.5
     // times as fast in panels), 60 of 40 x 400 dual 253 / 241 (primal 1.2 times);
     // FP32 rounds only with few rows: 1 of 5 x 12000 226 / 146, of 10 x 2000 1.06.
-    bool panel = no_room != nullptr;
-    for (int k = 0; k < count && panel; ++k)
-        panel = panel_smem(prec, m[k], n[k] + m[k] + 1, std::min(sms, kPanelMaxCtas),
-                           kPanelBatchK) <= kPanelBatchSmem;
+    bool panel = no_room != nullptr && panel_fits(count, m, n, prec, sms);
 
     // shapes: CTAs per LP from its tableau size, strips of whole sectors
     std::vector<int> M(count), N(count), G(count), W(count), sv(count);
@@ -855,10 +863,9 @@ extern "C" lp_err lp_batch_stats(double *kernel_ms, long long *pivots, int *ctas
 // Picks the batched launch shape (tableau elements per CTA of a group, and the
 // CTA size where the batch's kernel has a choice) for a batch by timing every
 // candidate on the batch itself (the best of two solves each, batched pivot
-// kernel time).  Results are cached in a
-// text file, one line "key group_elems threads kernel_ms" per batch
-// signature (count and a hash of the sorted shapes), so a serving process
-// tunes once per workload mix.
+// kernel time).  Results are cached in a text file, one line "key group_elems
+// threads kernel_ms" per kernel and batch signature (count and a hash of the
+// sorted shapes), so a serving process tunes once per workload mix.
 
 namespace {
 
@@ -905,11 +912,27 @@ extern "C" lp_err lp_batch_autotune(int count, const int *m, const int *n,
     lp_options o;
     if (opt) o = *opt; else lp_options_default(&o);
     if (count < 1 || !m || !n) return bfail(LP_ERR_INVALID_ARG, "lp_batch_autotune: empty batch");
-    char key[128];
-    snprintf(key, sizeof key, "fp64-c%d-%016llx", count, shape_signature(count, m, n));
+    // Batches that the panel kernel can take have a key of its own: a choice that
+    // was timed on the other kernel is none for it (1024 LPs 5.8 ms at 262144
+    // elements per CTA, 8.9 at 524288).
+    const int prec = o.precision == LP_FP32_REINV ? PREC_FP32 : PREC_FP64;
+    const unsigned long long sig = shape_signature(count, m, n);
+    char panel_key[128], key[128];
+    snprintf(panel_key, sizeof panel_key, "panel-%s-c%d-%016llx", prec == PREC_FP32 ? "fp32" : "fp64", count,
+             sig);
+    snprintf(key, sizeof key, "fp64-c%d-%016llx", count, sig);
     long long ge = 0;
-    int th = 0;
-    if (cache_lookup(cache_path, key, &ge, &th)) {
+    int th = 0, sms = 0;
+    bool hit = cache_lookup(cache_path, panel_key, &ge, &th);
+    if (!hit) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, o.device) != cudaSuccess) {
+            cudaGetLastError();
+            sms = 152;  // (a file is read without a device too)
+        }
+        if (panel_fits(count, m, n, prec, sms)) memcpy(key, panel_key, sizeof key);
+        else hit = cache_lookup(cache_path, key, &ge, &th);
+    }
+    if (hit) {
         *best = o;
         best->group_elems = ge;
         best->threads = th;
