@@ -796,11 +796,6 @@ lp_err reinvert(lp_handle *h, bool *singular, double *zmin, double *rmin) {
     CUDA_TRY(h, launch_reinv_solve(h->prec, h->dA, h->db, h->dc, h->sense, m, n, h->dbasis, h->rb,
                                    ns, h->dT, h->P, h->dx, h->dy, h->dobj, h->sms,
                                    h->opt.spin_timeout_cycles, s));
-    // the rows are rewritten from here on (rhs, objective row, the body's
-    // refresh, the dual rule's recovery): a -0 may be present
-    const int negz = 1;
-    CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, negz), &negz, sizeof negz,
-                                cudaMemcpyHostToDevice, s));
     ReinvCheck chk;
     CUDA_TRY(h, cudaMemcpyAsync(&chk, h->rb.chk, sizeof chk, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(h, cudaEventRecord(e1, s));
@@ -818,11 +813,20 @@ lp_err reinvert(lp_handle *h, bool *singular, double *zmin, double *rmin) {
     return LP_OK;
 }
 
+// What a reinversion leaves for the next launch: 1, rows were rewritten (rhs,
+// objective row, the dual rule's recovery) and a -0 may be present; 3, and the body
+// refreshed, its basic columns exact unit vectors.
+lp_err set_negz(lp_handle *h, int negz) {
+    CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, negz), &negz, sizeof negz,
+                                cudaMemcpyHostToDevice, h->stream));
+    return LP_OK;
+}
+
 // The FP32 tableau's constraint rows B^-1 [A I] recomputed from the FP64 data
 // for the basis of the last reinversion (lp_options.reinv_body), before the
 // tableau is pivoted again.
 lp_err refresh_body(lp_handle *h) {
-    if (h->prec != PREC_FP32 || !h->opt.reinv_body || h->region) return LP_OK;
+    if (h->prec != PREC_FP32 || !h->opt.reinv_body || h->region) return set_negz(h, 1);
     cudaStream_t s = h->stream;
     cudaEvent_t e0, e1;
     CUDA_TRY(h, cudaEventCreate(&e0));
@@ -845,11 +849,7 @@ lp_err refresh_body(lp_handle *h) {
         set_err(h, "reinversion: a wait of the body refresh ran out");
         return LP_ERR_CUDA;
     }
-    // the basic columns were written as exact unit vectors, +0 elsewhere
-    const int negz = 3;
-    CUDA_TRY(h, cudaMemcpyAsync((char *)h->ddesc + offsetof(LpDesc, negz), &negz, sizeof negz,
-                                cudaMemcpyHostToDevice, s));
-    return LP_OK;
+    return set_negz(h, 3);
 }
 
 // FP32 tableau with FP64 reinversion: pivot reinv_k pivots at a time in FP32,
@@ -946,8 +946,13 @@ lp_err solve_fp32(lp_handle *h) {
         else if (rule == 1 && !dfeas && pfeas) rule = 0;
         if ((e = refresh_body(h)) != LP_OK) return e;
     }
-    h->pdesc->status = final;
     if (final == LP_TIMEOUT) h->timed_out = true;
+    // (at the limit it was refreshed, after a timeout it has to be loaded again)
+    if (final != LP_TIMEOUT && final != LP_ITER_LIMIT) {
+        const lp_err e = set_negz(h, 1);
+        if (e != LP_OK) return e;
+    }
+    h->pdesc->status = final;
     CUDA_TRY(h, cudaMemcpyAsync(h->pobj, h->dobj, sizeof(double), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
     h->solved = true;

@@ -1106,52 +1106,27 @@ __global__ void oz_basic_kernel(const int *__restrict__ basis, int m, int *__res
     if (i < m) basic_row[basis[i]] = i;
 }
 
-// L = the constraints whose slack is basic, ascending; Lrow[r] = the row
-// where the slack of L[r] is basic (one CTA of 1024 threads).
-__global__ void __launch_bounds__(1024) oz_llist_kernel(const int *__restrict__ basic_row, int m,
-                                                        int n, int *__restrict__ L,
-                                                        int *__restrict__ Lrow) {
+// Two lists, a CTA of 1024 threads each.  Block 0: L = the constraints whose slack is
+// basic, ascending; Lrow[r] = the row where the slack of L[r] is basic.  Block 1:
+// grp = the groups of four tableau columns (of the first `cols`) that are not all
+// basic slacks, ascending, then -1 up to `cap`.
+__global__ void __launch_bounds__(1024) oz_lists_kernel(const int *__restrict__ basic_row, int m, int n,
+                                                        int *__restrict__ L, int *__restrict__ Lrow,
+                                                        int cols, int cap, int *__restrict__ grp) {
     __shared__ int scan[1024];
     const int tid = threadIdx.x, B = blockDim.x;
-    const int chunk = (m + B - 1) / B;
-    const int l0 = min(m, tid * chunk), l1 = min(m, l0 + chunk);
-    int cnt = 0;
-    for (int l = l0; l < l1; ++l) cnt += basic_row[n + l] >= 0;
-    scan[tid] = cnt;
-    __syncthreads();
-    for (int o = 1; o < B; o <<= 1) {
-        const int a = tid >= o ? scan[tid - o] : 0;
-        __syncthreads();
-        scan[tid] += a;
-        __syncthreads();
-    }
-    int k = scan[tid] - cnt;
-    for (int l = l0; l < l1; ++l) {
-        const int r = basic_row[n + l];
-        if (r >= 0) {
-            L[k] = l;
-            Lrow[k] = r;
-            ++k;
-        }
-    }
-}
-
-// grp = the groups of four tableau columns (of the first `cols`) that are not
-// all basic slacks, ascending, then -1 up to `cap` (one CTA of 1024 threads).
-__global__ void __launch_bounds__(1024) oz_groups_kernel(const int *__restrict__ basic_row, int n,
-                                                         int cols, int cap, int *__restrict__ grp) {
-    __shared__ int scan[1024];
-    const int tid = threadIdx.x, B = blockDim.x, total = (cols + 3) / 4;
-    const int chunk = (total + B - 1) / B;
-    const int g0 = min(total, tid * chunk), g1 = min(total, g0 + chunk);
-    auto kept = [&](int g) {
-        if (4 * g < n) return true;
+    const bool groups = blockIdx.x == 1;
+    const int total = groups ? (cols + 3) / 4 : m, chunk = (total + B - 1) / B;
+    const int e0 = min(total, tid * chunk), e1 = min(total, e0 + chunk);
+    auto kept = [&](int e) {
+        if (!groups) return basic_row[n + e] >= 0;
+        if (4 * e < n) return true;
         bool some = false;
-        for (int j = 4 * g; j < min(cols, 4 * g + 4); ++j) some |= basic_row[j] < 0;
+        for (int j = 4 * e; j < min(cols, 4 * e + 4); ++j) some |= basic_row[j] < 0;
         return some;
     };
     int cnt = 0;
-    for (int g = g0; g < g1; ++g) cnt += kept(g);
+    for (int e = e0; e < e1; ++e) cnt += kept(e);
     scan[tid] = cnt;
     __syncthreads();
     for (int o = 1; o < B; o <<= 1) {
@@ -1161,9 +1136,14 @@ __global__ void __launch_bounds__(1024) oz_groups_kernel(const int *__restrict__
         __syncthreads();
     }
     int k = scan[tid] - cnt;
-    for (int g = g0; g < g1; ++g)
-        if (kept(g) && k < cap) grp[k++] = g;
-    for (int e = scan[B - 1] + tid; e < cap; e += B) grp[e] = -1;
+    for (int e = e0; e < e1; ++e) {
+        if (!kept(e)) continue;
+        if (!groups) L[k] = e, Lrow[k] = basic_row[n + e];
+        else if (k < cap) grp[k] = e;
+        ++k;
+    }
+    if (groups)
+        for (int e = scan[B - 1] + tid; e < cap; e += B) grp[e] = -1;
 }
 
 // The other groups' columns, in all m rows: unit vectors.
@@ -1266,8 +1246,7 @@ cudaError_t oz_refresh_body(const double *A, const double *b, int sense, int m, 
     if ((e = cudaMemsetAsync(w.basic_row, 0xff, sizeof(int) * (size_t)(n + m), s)) != cudaSuccess)
         return e;
     oz_basic_kernel<<<(m + 255) / 256, 256, 0, s>>>(basis, m, w.basic_row);
-    oz_llist_kernel<<<1, 1024, 0, s>>>(w.basic_row, m, n, w.L, w.Lrow);
-    oz_groups_kernel<<<1, 1024, 0, s>>>(w.basic_row, n, cols, gcap, w.grp);
+    oz_lists_kernel<<<2, 1024, 0, s>>>(w.basic_row, m, n, w.L, w.Lrow, cols, gcap, w.grp);
     {
         const int gs = std::max(1, (cols + 3) / 4 - (n + 3) / 4), bx = (gs + 255) / 256;
         oz_unit_kernel<<<dim3(bx, std::max(1, std::min(m, 16 * sms / bx))), 256, 0, s>>>(

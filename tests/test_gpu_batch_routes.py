@@ -62,6 +62,12 @@ def test_few_wide_lps(dual):
     _solve(_lps([(12, 1100)] * 320, dual), PANEL)
 
 
+def test_one_lp_past_the_panel_kernels_shared_memory():
+    """It takes the whole batch with it."""
+    _solve(_lps([(400, 400), (2, 30000), (9, 20)]), PANEL)
+    _solve(_lps([(400, 400), (2, 50000), (9, 20)]), EVERY_PIVOT)
+
+
 NO_ROOM = """
 import sys
 sys.path[:0] = [%r, %r]
