@@ -13,9 +13,9 @@
 // panel_solve), so every LP's pivots and results are bit for bit those of
 // solving it alone.  Two CTAs of 256 threads per SM: one LP's selection chain
 // runs under another's panels.  1024 LPs of 32 to 1024 rows and columns: the
-// pivot kernel takes 5.8 ms (24 with the kernel that updates the tableau every
+// pivot kernel takes 6.1 ms (24 with the kernel that updates the tableau every
 // pivot; 5.6 ms is the FP64 time of the columns that change), at 262144 tableau
-// elements per CTA (6.7 ms at 131072, 8.9 at 524288); FP32 rounds 2.1 ms (8).
+// elements per CTA (6.5 ms at 131072, 6.3 at 524288); FP32 rounds 1.9 ms (8).
 
 #include <cuda_runtime.h>
 #include <stdarg.h>
@@ -912,9 +912,8 @@ extern "C" lp_err lp_batch_autotune(int count, const int *m, const int *n,
     lp_options o;
     if (opt) o = *opt; else lp_options_default(&o);
     if (count < 1 || !m || !n) return bfail(LP_ERR_INVALID_ARG, "lp_batch_autotune: empty batch");
-    // Batches that the panel kernel can take have a key of its own: a choice that
-    // was timed on the other kernel is none for it (1024 LPs 5.8 ms at 262144
-    // elements per CTA, 8.9 at 524288).
+    // Batches that the panel kernel can take have a key of their own: what was
+    // timed on the other kernel says nothing about it.
     const int prec = o.precision == LP_FP32_REINV ? PREC_FP32 : PREC_FP64;
     const unsigned long long sig = shape_signature(count, m, n);
     char panel_key[128], key[128];

@@ -30,8 +30,10 @@
 // Measured, 7858 x 16385 x 334 (13 of the 28 pairs not zero), clocks per tile of
 // 128 x 64: MMAs 15.8 K (50 each; reading their operands from shared memory
 // takes 48), the epilogue up to handing tensor memory back 5 K, waits for
-// operands 4.6 K (8.5 K with two B stages), 32.5 K in all (43 K before); the
-// epilogue's second half, 18 K, runs under the next tile's MMAs.
+// operands 4.6 K (8.5 K with two B stages), about 30 K in all.  The epilogue's
+// second half runs under the next tile's MMAs; where one K block makes them few
+// the epilogue alone bounds a tile: 14.9 K (28 K while each thread stored its own
+// row).
 //
 // The body refresh (FP32 mode, not in the paper; Sec. 2 Steps 4-5 produce the
 // tableau B^-1 [A I b] that it recomputes): with S the structural basic

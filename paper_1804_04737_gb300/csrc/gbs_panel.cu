@@ -25,11 +25,11 @@
 // run on eight more warps and a second buffer while the next one's pivots are
 // selected (OV below): the chain takes about 9 us then, the panel's time is
 // hidden.  Measured, FP64, us per pivot, against the kernels that update
-// everything every one or two pivots: 256^2 6.9 (was 9.3), 501 x 703 of the
-// paper's family 6.6 (10.2), 512 x 4096 8.6 (10.8; in turn 10.9), 4096 x 512
-// 9.7 (42; 10.3), 2048^2 10.3 (22.4; 13.7), its dual form 12.3 (22.9; 16.1),
-// 4096^2 33 (59; 36), 8192^2 118 (136; overlapped 119; 107 is its fmas at the
-// FP64 peak); FP32 8192^2 16 (70).  In turn, panels of 8 pivots instead of 16
+// everything every one or two pivots: 64^2 6.4, 256^2 7.0 (was 9.3), 501 x 703 of
+// the paper's family 6.7 (10.2), 512 x 4096 8.6 (10.1; in turn 10.9), 4096 x 512
+// 9.7 (41; 10.3), 2048^2 10.3 (21.6; 13.7), its dual form 12.3 (22.9; 16.1),
+// 4096^2 33 (58; 36), 8192^2 118 (136; overlapped 119; 107 is its fmas at the
+// FP64 peak); FP32 8192^2 18 in launches of 50 pivots, 16 of 200 (70).  In turn, panels of 8 pivots instead of 16
 // were 1 to 4% slower from 512 x 4096 up; overlapped, four or six warps for the
 // panels were slower than eight from 2048^2 up (13.2 and 10.4 us).
 //
@@ -204,8 +204,9 @@ struct DivisorOf<float> {
 // a relative 2^-20 of the quotient, whose order as integers is the floats'
 // order, for operands with exponents within 2^+-60 (the quotient is then a
 // normal float); kWide marks operands outside, which have to be divided
-// exactly.  A row whose exactly rounded ratio is the smallest has a key at
-// most kNear above the smallest key (a relative 2^-15 or more), so rows
+// exactly.  kNear steps of a key are a relative 2^-16 (significand near 2) to
+// 2^-15 (near 1), more than twice a key's error: a row whose exactly rounded
+// ratio is the smallest has a key at most kNear above the smallest key, so rows
 // further off need no division.
 constexpr unsigned kNone = 0xffffffffu;  // not a candidate
 constexpr unsigned kNear = 256;
@@ -1635,8 +1636,9 @@ PivotShape choose_panel_shape(int prec, int M, int N, int sms, int ctas, int dua
     PivotShape sh;
     const int m = M - 1;
     // Default grid: every SM, on small LPs one CTA per two rows or 32 columns,
-    // whichever gives more (one row per CTA measured no faster: 64^2 6.7 us per
-    // pivot on 16 to 152 CTAs, 256^2 7.2 on 114 and on 152).
+    // whichever gives more (one row per CTA measured no faster: 64^2 6.4 us per
+    // pivot on 32 CTAs, 6.5 on 16 and 64, 6.7 on 152, 6.8 on one; 256^2 7.1 on 114
+    // and on 152).
     int G = ctas > 0 ? ctas : std::max((m + 1) / 2, (N + 31) / 32);
     G = std::min(G, std::min(sms, kPanelMaxCtas));
     G = std::max(1, std::min(G, N));
