@@ -1090,6 +1090,11 @@ bool engine_solo(lp_server *sv) {
     lp_err verdict = LP_OK, e = LP_OK;
     lp_handle *h = nullptr;
     bool spilled = false;
+    // FP64 with spill_pivots: slices of spill_pivots pivots (an FP64 solve
+    // cut into calls makes the same pivots, bit for bit); after a slice, when
+    // any request is waiting, the LP is spilled and goes to the back of the
+    // queue
+    const bool sliced = sv->spill_pivots > 0 && !sv->fp32;
     char why[160] = {0};
     if (bneg) {
         verdict = LP_ERR_INFEASIBLE_START;
@@ -1124,14 +1129,11 @@ bool engine_solo(lp_server *sv) {
         }
         h = sv->solo;
         if (e == LP_OK) e = handle_bind_region(h, sv->arena_dev + off, bytes);
+        // (the load chooses kernels by it; the handle has the last LP's slice)
+        if (sliced) handle_set_max_iters(h, std::min(sv->spill_pivots, sv->opt.max_iters));
         if (e == LP_OK) e = lp_load(h, m, n, A, b, c, (lp_sense)r->sense);
         if (e == LP_OK) r->resident_from = 0;
     }
-    // FP64 with spill_pivots: slices of spill_pivots pivots (an FP64 solve
-    // cut into calls makes the same pivots, bit for bit); after a slice, when
-    // any request is waiting, the LP is spilled and goes to the back of the
-    // queue
-    const bool sliced = sv->spill_pivots > 0 && !sv->fp32;
     while (h && e == LP_OK && verdict == LP_OK) {
         if (sliced) handle_set_max_iters(h, std::min(sv->spill_pivots, sv->opt.max_iters - iters));
         e = lp_solve(h);
